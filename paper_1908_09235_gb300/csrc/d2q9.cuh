@@ -227,9 +227,33 @@ __device__ __forceinline__ float r_fma(float a, float b, float c) { return __fma
 __device__ __forceinline__ double r_fma(double a, double b, double c) { return __fma_rn(a, b, c); }
 __device__ __forceinline__ float2 r_fma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
 
+// FP64 psi with the node's 1/rho, which its collision needs too: one reciprocal serves both, since
+// the FP64 pipe bounds the step (a reciprocal or division costs it about as much as eight
+// additions).  Carnahan-Starling: r = 1 / (rho (1 - eta)^3) gives 1/rho = (1 - eta)^3 r and
+// 1/(1 - eta)^3 = rho r.
+template <int EOS>
+__device__ __forceinline__ double psi_inv(const Consts<double>& k, double rho, double& inv_rho) {
+  if constexpr (EOS == LBM_EOS_EXP) {
+    inv_rho = q_rcp(rho);
+    return r_mul(k.psi0, q_exp(r_mul(-k.rho0, inv_rho)));
+  } else {
+    const double eta = r_mul(k.b4, rho);
+    const double om = r_sub(1.0, eta);
+    const double num = r_fma(eta, r_fma(eta, om, 1.0), 1.0);
+    const double om3 = r_mul(r_mul(om, om), om);
+    const double r = q_rcp(r_mul(rho, om3));
+    inv_rho = r_mul(om3, r);
+    const double inner = r_fma(r_mul(k.RT, num), r_mul(rho, r), r_fma(-k.a, rho, -1.0 / 3.0));
+    return q_sqrt(r_mul(r_mul(rho, k.two_over_G), inner));
+  }
+}
+
 template <typename C, int EOS, typename L>
 __device__ __forceinline__ L psi_of(const Consts<C>& k, L rho) {
-  if constexpr (EOS == LBM_EOS_EXP) {
+  if constexpr (EOS != LBM_EOS_NONE && sizeof(C) == 8) {
+    double inv_rho;
+    return psi_inv<EOS>(k, rho, inv_rho);
+  } else if constexpr (EOS == LBM_EOS_EXP) {
     return r_mul(splat<L>(k.psi0), q_exp(r_mul(splat<L>(C(-1)), q_div(splat<L>(k.rho0), rho))));
   } else if constexpr (EOS == LBM_EOS_CS) {
     // p = rho R T (1 + eta + eta^2 - eta^3) / (1 - eta)^3 - a rho^2,  eta = b rho / 4, so
@@ -246,6 +270,16 @@ __device__ __forceinline__ L psi_of(const Consts<C>& k, L rho) {
   } else {
     return splat<L>(C(0));
   }
+}
+
+// psi of a node and what its collision reuses: 1/rho for FP64 (unused by FP32 arithmetic, whose
+// hardware reciprocal is cheaper than keeping the value).
+template <typename C, int EOS, typename L>
+__device__ __forceinline__ L psi_own(const Consts<C>& k, L rho, L& inv_rho) {
+  if constexpr (EOS != LBM_EOS_NONE && sizeof(C) == 8)
+    return psi_inv<EOS>(k, rho, inv_rho);
+  else
+    return psi_of<C, EOS>(k, rho);
 }
 
 }  // namespace lbm

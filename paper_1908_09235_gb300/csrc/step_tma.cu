@@ -155,7 +155,7 @@ __global__ void __launch_bounds__(TX* TYM, 2)
 
     // phase 1 from the stage: own nodes and the ring (lattices of at least 64 x 64: one wrap)
     C f[RYT][9];
-    C rho[RYT];
+    C rho[RYT], inv[RYT];
     uint8_t fl[RYT];
 #pragma unroll
     for (int r = 0; r < RYT; ++r) {
@@ -192,7 +192,7 @@ __global__ void __launch_bounds__(TX* TYM, 2)
     }
     __syncthreads();
     tile_phase2<float, EOS, false, RYT, TYM>(p, fb, rho_m, ux_m, uy_m, x0, y0, psi_s, f, rho,
-                                             fl);
+                                             inv, fl);
     __syncthreads();  // the stage and psi_s are free for the next tile
   }
 }

@@ -468,7 +468,7 @@ __global__ void __launch_bounds__(VW* Vec<S>::VH, Vec<S>::kBlocks)
     load_own();
   }
 
-  L rho[NP];
+  L rho[NP], inv[NP];
 #pragma unroll
   for (int q = 0; q < NP; ++q) {
     const L r = density_of<DEV>(rho_ref, f[q]);
@@ -477,7 +477,7 @@ __global__ void __launch_bounds__(VW* Vec<S>::VH, Vec<S>::kBlocks)
     for (int e = 0; e < W; ++e) re[e] = (fl[W * q + e] & FLAG_SOLID) ? C(1) : el(r, e);
     rho[q] = pack<L>(re[0], re[W - 1]);
     if constexpr (PSI) {
-      const L ps = psi_of<C, EOS>(k, rho[q]);
+      const L ps = psi_own<C, EOS>(k, rho[q], inv[q]);
 #pragma unroll
       for (int e = 0; e < W; ++e)
         if (lane_ok)
@@ -567,7 +567,7 @@ __global__ void __launch_bounds__(VW* Vec<S>::VH, Vec<S>::kBlocks)
     }
     const int x = x0 + V * lane + W * q;
     L st[9], ux, uy;
-    collide_node<S, EOS, L>(p, k, f[q], rho[q], d13, d24, d57, d86, psic,
+    collide_node<S, EOS, L>(p, k, f[q], rho[q], inv[q], d13, d24, d57, d86, psic,
                             pack<L>(C(x), C(x + W - 1)), splat<L>(C(yo)), st, ux, uy);
 #pragma unroll
     for (int e = 0; e < W; ++e) {

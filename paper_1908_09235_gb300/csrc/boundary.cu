@@ -239,11 +239,11 @@ __device__ __forceinline__ void boundary_group(const DevParams& p, int b, int k,
   // macro arrays, the lattice values, the FP64 carry) was written by the kernels before this
   // one.  Launched as a programmatic dependent of the step kernel, the pass waits here for that
   // grid to complete and its writes to be visible; otherwise the wait returns at once.
-  asm volatile("griddepcontrol.wait;" ::: "memory");
+  pdl_wait();
   if (act) {
-    rho_b = rhoT[LBM_CHK(n, N)];
-    ubx = uxT[n];
-    uby = uyT[n];
+    rho_b = __ldcg(rhoT + LBM_CHK(n, N));
+    ubx = __ldcg(uxT + n);
+    uby = __ldcg(uyT + n);
   }
   // second loads: lattice values (deviations d_ for the FP32 formats; f = d_ + w rho_ref)
   const T w = wgt<T>(a);
@@ -255,8 +255,8 @@ __device__ __forceinline__ void boundary_group(const DevParams& p, int b, int k,
     if (x2 >= 0) X2 = Pop<S>::load_t((kind & kFromA) ? L.src : L.dst, x2, N) + wr;
     if (kind & kGhost) {
       if (uf >= 0) {
-        usx = uxT[LBM_CHK(uf, N)];
-        usy = uyT[uf];
+        usx = __ldcg(uxT + LBM_CHK(uf, N));
+        usy = __ldcg(uyT + uf);
       } else {
         usx = cus * ubx;
         usy = cus * uby;
@@ -307,7 +307,7 @@ __device__ __forceinline__ void boundary_group(const DevParams& p, int b, int k,
       // exact FP64 imbalance of the stored deviations (the w rho_ref parts cancel)
       const double dm = group8_sum(act ? double(fo_d) - double(in_d) : 0.0, mask);
       if (lane0) {
-        const double want = double(f0_d) + dm + carry[b];
+        const double want = double(f0_d) + dm + __ldcg(carry + b);
         if (want != double(f0_d)) {
           const T st = Pop<S>::store_t(L.dst, n, N, T(want));
           carry[b] = want - double(st);
@@ -324,6 +324,43 @@ __device__ __forceinline__ void boundary_group(const DevParams& p, int b, int k,
   }
 }
 
+// Channel ends (Sec. 4.2), after streaming and the wall pass; one thread per row j.  Inlet
+// i = 0: the populations entering from the left (1, 5, 8) follow from the prescribed velocity
+// (u_in, 0) and the known ones by Zou and He's rule:
+//   rho = (f0 + f2 + f4 + 2 (f3 + f6 + f7)) / (1 - u_in),  f1 = f3 + 2/3 rho u_in,
+//   f5 = f7 - (f2 - f4)/2 + rho u_in / 6,  f8 = f6 + (f2 - f4)/2 + rho u_in / 6.
+// Outlet i = nx - 1 (fully developed flow): the populations entering from the right (3, 6, 7)
+// equal those of column nx - 2.  FP64 arithmetic on the full populations (deviation + w rho_ref).
+template <typename S>
+__device__ __forceinline__ void open_row(const DevParams& p, int j, void* __restrict__ fb,
+                                         const uint8_t* __restrict__ flags, double u_in) {
+  const int nx = p.nx, N = p.N;
+  const double rr = p.rho_ref;
+  const bool in = j < p.ny;
+  const int n0 = in ? j * nx : 0, n1 = n0 + nx - 1;
+  const bool fluid0 = in && !(flags[n0] & FLAG_SOLID), fluid1 = in && !(flags[n1] & FLAG_SOLID);
+  pdl_wait();
+  auto get = [&](int a, int n) { return Pop<S>::load_e(fb, a * N + n, N) + wgt<double>(a) * rr; };
+  auto put = [&](int a, int n, double v) { Pop<S>::store_e(fb, a * N + n, N, v - wgt<double>(a) * rr); };
+  if (fluid0) {
+    const double f0 = get(0, n0), f2 = get(2, n0), f3 = get(3, n0), f4 = get(4, n0);
+    const double f6 = get(6, n0), f7 = get(7, n0);
+    const double rho = (f0 + f2 + f4 + 2.0 * (f3 + f6 + f7)) / (1.0 - u_in);
+    put(1, n0, f3 + 2.0 / 3.0 * rho * u_in);
+    put(5, n0, f7 - 0.5 * (f2 - f4) + rho * u_in / 6.0);
+    put(8, n0, f6 + 0.5 * (f2 - f4) + rho * u_in / 6.0);
+  }
+  if (fluid1) {
+    // copies of stored values: no rounding for any format
+    Pop<S>::store_e(fb, 3 * N + n1, N, Pop<S>::load_e(fb, 3 * N + n1 - 1, N));
+    Pop<S>::store_e(fb, 6 * N + n1, N, Pop<S>::load_e(fb, 6 * N + n1 - 1, N));
+    Pop<S>::store_e(fb, 7 * N + n1, N, Pop<S>::load_e(fb, 7 * N + n1 - 1, N));
+  }
+}
+
+// The wall pass: 8 lanes per boundary node.  CTAs from wall_ctas on (launched only in channel mode
+// when no boundary node reads or writes what the channel ends touch) do the channel ends, one
+// thread per row, so that the two need one launch.
 template <typename S>
 __global__ void __launch_bounds__(128) boundary_kernel(DevParams p, int nb,
                                                        const int32_t* __restrict__ bnode,
@@ -334,45 +371,24 @@ __global__ void __launch_bounds__(128) boundary_kernel(DevParams p, int nb,
                                                        const double* __restrict__ ux_m,
                                                        const double* __restrict__ uy_m,
                                                        double* __restrict__ carry,
-                                                       double* __restrict__ force) {
+                                                       double* __restrict__ force, int wall_ctas,
+                                                       const uint8_t* __restrict__ flags,
+                                                       double u_in) {
+  if ((int)blockIdx.x >= wall_ctas) {
+    open_row<S>(p, (blockIdx.x - wall_ctas) * blockDim.x + threadIdx.x, L.dst, flags, u_in);
+    return;
+  }
   const int gt = blockIdx.x * blockDim.x + threadIdx.x;
   const int b = gt >> 3;
   boundary_group<S>(p, b, gt & 7, b < nb, bnode, boff, ldir, r, L, rho_m, ux_m, uy_m, carry,
                     force, 0xffffffffu);
 }
 
-// Channel ends (Sec. 4.2), after streaming and the wall pass; one thread per row j.  Inlet
-// i = 0: the populations entering from the left (1, 5, 8) follow from the prescribed velocity
-// (u_in, 0) and the known ones by Zou and He's rule:
-//   rho = (f0 + f2 + f4 + 2 (f3 + f6 + f7)) / (1 - u_in),  f1 = f3 + 2/3 rho u_in,
-//   f5 = f7 - (f2 - f4)/2 + rho u_in / 6,  f8 = f6 + (f2 - f4)/2 + rho u_in / 6.
-// Outlet i = nx - 1 (fully developed flow): the populations entering from the right (3, 6, 7)
-// equal those of column nx - 2.  FP64 arithmetic on the full populations (deviation + w rho_ref).
 template <typename S>
-__global__ void open_x_kernel(DevParams p, void* __restrict__ fb,
-                              const uint8_t* __restrict__ flags, double u_in) {
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= p.ny) return;
-  const int nx = p.nx, N = p.N;
-  const double rr = p.rho_ref;
-  auto get = [&](int a, int n) { return Pop<S>::load_e(fb, a * N + n, N) + wgt<double>(a) * rr; };
-  auto put = [&](int a, int n, double v) { Pop<S>::store_e(fb, a * N + n, N, v - wgt<double>(a) * rr); };
-  const int n0 = j * nx;
-  if (!(flags[n0] & FLAG_SOLID)) {
-    const double f0 = get(0, n0), f2 = get(2, n0), f3 = get(3, n0), f4 = get(4, n0);
-    const double f6 = get(6, n0), f7 = get(7, n0);
-    const double rho = (f0 + f2 + f4 + 2.0 * (f3 + f6 + f7)) / (1.0 - u_in);
-    put(1, n0, f3 + 2.0 / 3.0 * rho * u_in);
-    put(5, n0, f7 - 0.5 * (f2 - f4) + rho * u_in / 6.0);
-    put(8, n0, f6 + 0.5 * (f2 - f4) + rho * u_in / 6.0);
-  }
-  const int n1 = j * nx + nx - 1;
-  if (!(flags[n1] & FLAG_SOLID)) {
-    // copies of stored values: no rounding for any format
-    Pop<S>::store_e(fb, 3 * N + n1, N, Pop<S>::load_e(fb, 3 * N + n1 - 1, N));
-    Pop<S>::store_e(fb, 6 * N + n1, N, Pop<S>::load_e(fb, 6 * N + n1 - 1, N));
-    Pop<S>::store_e(fb, 7 * N + n1, N, Pop<S>::load_e(fb, 7 * N + n1 - 1, N));
-  }
+__global__ void __launch_bounds__(128) open_x_kernel(DevParams p, void* __restrict__ fb,
+                                                     const uint8_t* __restrict__ flags,
+                                                     double u_in) {
+  open_row<S>(p, blockIdx.x * blockDim.x + threadIdx.x, fb, flags, u_in);
 }
 
 // Boundary nodes of many lattices: items are (domain, boundary node); a persistent grid of
@@ -408,28 +424,22 @@ __global__ void batch_advance_kernel(BatchDomain* __restrict__ doms, int n, int*
   }
 }
 
+// CTAs of one warp while that leaves at most four on an SM: a group is a chain of dependent loads
+// and (FP64) of narrow-pipe operations, so a few warps are best spread over as many SMs.
+unsigned wall_threads(long long threads) { return threads <= 32LL * 152 * 4 ? 32 : 128; }
+
 template <typename S>
 cudaError_t launch_b(const DevParams& p, int nb, const int32_t* bnode, const int32_t* boff,
                      const uint8_t* ldir, LinkRecipe r, const void* fa, void* fb,
                      const double* rho_m, const double* ux_m, const double* uy_m, double* carry,
-                     double* force, cudaStream_t s) {
+                     double* force, const uint8_t* open_flags, double u_in, cudaStream_t s) {
   Lat<S> L{fa, fb, p.N, p.rho_ref};  // rho_ref also in p.k<T>() for the FP32 formats
   const long long threads = 8LL * nb;
-  // a programmatic dependent of the kernel before it in the stream (the step kernel): its CTAs
-  // may start, and load their link records, while that grid drains; they wait for it before
-  // reading anything it wrote (griddepcontrol.wait in boundary_group)
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3((unsigned)((threads + 127) / 128));
-  cfg.blockDim = dim3(128);
-  cfg.dynamicSmemBytes = 0;
-  cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, boundary_kernel<S>, p, nb, bnode, boff, ldir, r, L, rho_m, ux_m,
-                            uy_m, carry, force);
+  const unsigned nt = wall_threads(threads + (open_flags ? p.ny : 0));
+  const unsigned wall = (unsigned)((threads + nt - 1) / nt);
+  const unsigned ends = open_flags ? (p.ny + nt - 1) / nt : 0;
+  return launch_pdl(boundary_kernel<S>, dim3(wall + ends), dim3(nt), s, p, nb, bnode, boff, ldir,
+                    r, L, rho_m, ux_m, uy_m, carry, force, (int)wall, open_flags, u_in);
 }
 
 size_t align256(size_t v) { return (v + 255) / 256 * 256; }
@@ -509,26 +519,28 @@ cudaError_t launch_batch_advance(BatchDomain* doms, int n_doms, int* claim, cuda
 cudaError_t launch_boundary(int precision, const DevParams& p, int nb, const int32_t* bnode,
                             const int32_t* boff, const uint8_t* ldir, LinkRecipe r,
                             const void* fa, void* fb, const double* rho_m, const double* ux_m,
-                            const double* uy_m, double* carry, double* force, cudaStream_t s) {
+                            const double* uy_m, double* carry, double* force,
+                            const uint8_t* open_flags, double u_in, cudaStream_t s) {
   if (nb <= 0) return cudaSuccess;
   if (precision == LBM_FP32_DEV)
-    return launch_b<float>(p, nb, bnode, boff, ldir, r, fa, fb, rho_m, ux_m, uy_m, carry, force, s);
+    return launch_b<float>(p, nb, bnode, boff, ldir, r, fa, fb, rho_m, ux_m, uy_m, carry, force,
+                           open_flags, u_in, s);
   if (precision == LBM_FP16_DEV)
     return launch_b<__half>(p, nb, bnode, boff, ldir, r, fa, fb, rho_m, ux_m, uy_m, carry, force,
-                            s);
-  return launch_b<double>(p, nb, bnode, boff, ldir, r, fa, fb, rho_m, ux_m, uy_m, carry, force, s);
+                            open_flags, u_in, s);
+  return launch_b<double>(p, nb, bnode, boff, ldir, r, fa, fb, rho_m, ux_m, uy_m, carry, force,
+                          open_flags, u_in, s);
 }
 
 cudaError_t launch_open_x(int precision, const DevParams& p, void* fb, const uint8_t* flags,
                           double u_in, cudaStream_t s) {
-  const unsigned grid = (unsigned)((p.ny + 127) / 128);
+  const unsigned nt = wall_threads(p.ny);
+  const dim3 grid((p.ny + nt - 1) / nt);
   if (precision == LBM_FP32_DEV)
-    open_x_kernel<float><<<grid, 128, 0, s>>>(p, fb, flags, u_in);
-  else if (precision == LBM_FP16_DEV)
-    open_x_kernel<__half><<<grid, 128, 0, s>>>(p, fb, flags, u_in);
-  else
-    open_x_kernel<double><<<grid, 128, 0, s>>>(p, fb, flags, u_in);
-  return cudaGetLastError();
+    return launch_pdl(open_x_kernel<float>, grid, dim3(nt), s, p, fb, flags, u_in);
+  if (precision == LBM_FP16_DEV)
+    return launch_pdl(open_x_kernel<__half>, grid, dim3(nt), s, p, fb, flags, u_in);
+  return launch_pdl(open_x_kernel<double>, grid, dim3(nt), s, p, fb, flags, u_in);
 }
 
 }  // namespace lbm

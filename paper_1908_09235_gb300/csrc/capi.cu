@@ -87,20 +87,26 @@ cudaError_t launch_bulk(lbm_ctx* c, cudaStream_t s, int cur) {
                      c->uy_m, false, s, c->kernel_path, c->err_flag);
 }
 
-lbm_status launch_one_step(lbm_ctx* c, cudaStream_t s, int cur) {
-  const void* fa = c->f[cur];
+// The wall pass and, in channel mode, the channel ends of a step from lattice cur.
+lbm_status launch_walls(lbm_ctx* c, cudaStream_t s, int cur) {
   void* fb = c->f[1 - cur];
-  cudaError_t e = launch_bulk(c, s, cur);
-  if (e != cudaSuccess) return cuda_fail(c, e, "step kernel launch");
-  e = launch_boundary(c->precision, c->p, (int)c->nb, c->bnode, c->boff, c->ldir, c->recipe, fa,
-                      fb, c->rho_m, c->ux_m, c->uy_m, c->carry,
-                      c->track_force ? c->force : nullptr, s);
+  const bool together = c->open_x && c->ends_with_wall && c->nb > 0;
+  cudaError_t e = launch_boundary(c->precision, c->p, (int)c->nb, c->bnode, c->boff, c->ldir,
+                                  c->recipe, c->f[cur], fb, c->rho_m, c->ux_m, c->uy_m, c->carry,
+                                  c->track_force ? c->force : nullptr,
+                                  together ? c->flags : nullptr, c->u_in, s);
   if (e != cudaSuccess) return cuda_fail(c, e, "boundary kernel launch");
-  if (c->open_x) {
+  if (c->open_x && !together) {
     e = launch_open_x(c->precision, c->p, fb, c->flags, c->u_in, s);
     if (e != cudaSuccess) return cuda_fail(c, e, "channel-end kernel launch");
   }
   return LBM_OK;
+}
+
+lbm_status launch_one_step(lbm_ctx* c, cudaStream_t s, int cur) {
+  cudaError_t e = launch_bulk(c, s, cur);
+  if (e != cudaSuccess) return cuda_fail(c, e, "step kernel launch");
+  return launch_walls(c, s, cur);
 }
 
 lbm_status build_graph(lbm_ctx* c, int parity) {
@@ -126,6 +132,18 @@ lbm_status build_graph(lbm_ctx* c, int parity) {
 }
 
 bool is_fin(double v) { return std::isfinite(v); }
+
+// The wall pass and the channel ends touch different nodes: every solid body is a disc, so the
+// wall pass reads and writes nodes within its box widened by 1 + 2 (a boundary node, and two
+// nodes behind it); the ends touch columns 0, nx - 2 and nx - 1.
+bool ends_clear_of_walls(const GeomParams& g) {
+  if (g.wall_q_lo > 0.0 || g.wall_q_hi > 0.0) return false;
+  for (int k = 0; k < g.n_circles; ++k)
+    if (g.c[k].outside || g.c[k].cx - g.c[k].r - 4.0 < 1.0 ||
+        g.c[k].cx + g.c[k].r + 4.0 > g.nx - 3.0)
+      return false;
+  return true;
+}
 
 }  // namespace
 
@@ -262,6 +280,7 @@ lbm_status lbm_create(const lbm_geometry* geo, const lbm_eos* eos, double tau, i
   const size_t N = (size_t)p.N;
   const int gblocks = geom_num_blocks(p.N);
   c->ledger_blocks = ledger_num_blocks(p.N);
+  c->ends_with_wall = ends_clear_of_walls(g);
   size_t bytes = 2 * align_up(c->lattice_bytes) + align_up((N + 3) / 4 * 4) +
                  3 * align_up(N * 8) + align_up(c->ledger_blocks * 8) + align_up(8) +
                  align_up(sizeof(int)) + align_up(gblocks * sizeof(int2)) + align_up(16);
@@ -469,16 +488,7 @@ lbm_status lbm_step_timed(lbm_ctx* c, int32_t n, double* ms_step, double* ms_bnd
     cudaError_t e = launch_bulk(c, c->stream, cur);
     if (e != cudaSuccess) st = cuda_fail(c, e, "step kernel launch");
     if (st == LBM_OK) cudaEventRecord(ev[2 * k + 1], c->stream);
-    if (st == LBM_OK) {
-      e = launch_boundary(c->precision, c->p, (int)c->nb, c->bnode, c->boff, c->ldir, c->recipe,
-                          c->f[cur], c->f[1 - cur], c->rho_m, c->ux_m, c->uy_m, c->carry,
-                          c->track_force ? c->force : nullptr, c->stream);
-      if (e != cudaSuccess) st = cuda_fail(c, e, "boundary kernel launch");
-    }
-    if (st == LBM_OK && c->open_x) {
-      e = launch_open_x(c->precision, c->p, c->f[1 - cur], c->flags, c->u_in, c->stream);
-      if (e != cudaSuccess) st = cuda_fail(c, e, "channel-end kernel launch");
-    }
+    if (st == LBM_OK) st = launch_walls(c, c->stream, cur);
     if (st == LBM_OK) cudaEventRecord(ev[2 * k + 2], c->stream);
     c->cur = 1 - cur;
     ++c->steps;

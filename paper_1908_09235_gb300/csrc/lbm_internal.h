@@ -153,8 +153,10 @@ cudaError_t launch_link_setup(const DevParams& p, int nb, const int32_t* bnode,
 cudaError_t launch_boundary(int precision, const DevParams& p, int nb, const int32_t* bnode,
                             const int32_t* boff, const uint8_t* ldir, LinkRecipe r,
                             const void* fa, void* fb, const double* rho_m, const double* ux_m,
-                            const double* uy_m, double* carry, double* force, cudaStream_t s);
-// force: per boundary node (fx, fy) of the momentum exchange with the walls, or nullptr
+                            const double* uy_m, double* carry, double* force,
+                            const uint8_t* open_flags, double u_in, cudaStream_t s);
+// open_flags (with nb > 0): the node flags, to do the channel ends in the same launch (only where
+// they and the wall pass touch different nodes), or nullptr.  force: per boundary node (fx, fy) of the momentum exchange with the walls, or nullptr
 // Channel ends (velocity inlet at column 0, fully developed outlet at column nx - 1)
 cudaError_t launch_open_x(int precision, const DevParams& p, void* fb, const uint8_t* flags,
                           double u_in, cudaStream_t s);
@@ -241,6 +243,7 @@ struct lbm_ctx {
   bool track_force = false;   // the wall pass fills `force` (lbm_options.track_force, inflow)
   bool open_x = false;        // channel mode (lbm_set_inflow)
   double u_in = 0.0;
+  bool ends_with_wall = false;  // the channel ends can share the wall pass's launch
   lbm::LinkRecipe recipe{};
   double* partials = nullptr;
   double* mass_out = nullptr;

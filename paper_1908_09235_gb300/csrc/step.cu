@@ -27,16 +27,16 @@ constexpr int tile_ctas() {
   return sizeof(S) == 8 ? 2 : (sizeof(S) == 4 && RY == 4 ? 3 : 4);
 }
 
-template <typename S, int EOS, bool FIELDS>
-__global__ void __launch_bounds__(TX* TYT, tile_ctas<S, StoreTraits<S>::RY>())
+// TXN x TYN threads, RY rows per thread.
+template <typename S, int EOS, bool FIELDS, int TXN, int TYN, int RY>
+__global__ void __launch_bounds__(TXN* TYN, tile_ctas<S, RY>() * (TX * TYT) / (TXN * TYN))
     step_kernel(DevParams p, const void* __restrict__ fa, void* __restrict__ fb,
                 const uint8_t* __restrict__ flags, double* __restrict__ rho_m,
                 double* __restrict__ ux_m, double* __restrict__ uy_m) {
   using C = typename StoreTraits<S>::C;
-  constexpr int RY = StoreTraits<S>::RY;
-  __shared__ C psi_s[TYT * RY + 2][TX + 2];
-  step_tile<S, EOS, FIELDS, RY>(p, fa, fb, flags, rho_m, ux_m, uy_m, blockIdx.x * TX,
-                                blockIdx.y * TYT * RY, psi_s);
+  __shared__ C psi_s[TYN * RY + 2][TXN + 2];
+  step_tile<S, EOS, FIELDS, RY, TYN, TXN, true>(p, fa, fb, flags, rho_m, ux_m, uy_m,
+                                                blockIdx.x * TXN, blockIdx.y * TYN * RY, psi_s);
 }
 
 // Many lattices in one launch: a persistent grid works through a queue of tiles (domain, x0,
@@ -75,18 +75,27 @@ __global__ void __launch_bounds__(TX* TYT, tile_ctas<S, RY>())
 }
 
 
+template <typename S, int EOS, int TXN, int TYN, int RY>
+cudaError_t launch_shape(const DevParams& p, const void* fa, void* fb, const uint8_t* flags,
+                         double* rho_m, double* ux_m, double* uy_m, bool fields_only,
+                         cudaStream_t s) {
+  constexpr int TH = TYN * RY;
+  const dim3 block(TXN, TYN), grid((p.nx + TXN - 1) / TXN, (p.ny + TH - 1) / TH);
+  if (fields_only) {
+    step_kernel<S, EOS, true, TXN, TYN, RY>
+        <<<grid, block, 0, s>>>(p, fa, fb, flags, rho_m, ux_m, uy_m);
+    return cudaGetLastError();
+  }
+  return launch_pdl(step_kernel<S, EOS, false, TXN, TYN, RY>, grid, block, s, p, fa, fb, flags,
+                    rho_m, ux_m, uy_m);
+}
+
 template <typename S, int EOS>
 cudaError_t launch_t(const DevParams& p, const void* fa, void* fb, const uint8_t* flags,
                      double* rho_m, double* ux_m, double* uy_m, bool fields_only,
                      cudaStream_t s) {
-  constexpr int TH = TYT * StoreTraits<S>::RY;
-  dim3 block(TX, TYT);
-  dim3 grid((p.nx + TX - 1) / TX, (p.ny + TH - 1) / TH);
-  if (fields_only)
-    step_kernel<S, EOS, true><<<grid, block, 0, s>>>(p, fa, fb, flags, rho_m, ux_m, uy_m);
-  else
-    step_kernel<S, EOS, false><<<grid, block, 0, s>>>(p, fa, fb, flags, rho_m, ux_m, uy_m);
-  return cudaGetLastError();
+  return launch_shape<S, EOS, TX, TYT, StoreTraits<S>::RY>(p, fa, fb, flags, rho_m, ux_m, uy_m,
+                                                          fields_only, s);
 }
 
 template <typename S>

@@ -204,12 +204,12 @@ __device__ __forceinline__ void collide_node(const DevParams& p,
 // psi_s (complete: the caller has synchronised the CTA).  Writes the moments of FLAG_MACRO nodes
 // for the wall pass (FIELDS: the moments of every node instead) and pushes (Eq. 3) the
 // post-collision populations to x + e_a of fb.
-template <typename S, int EOS, bool FIELDS, int RY, int TYN = TYT>
+template <typename S, int EOS, bool FIELDS, int RY, int TYN = TYT, int TXN = TX>
 __device__ __forceinline__ void tile_phase2(const DevParams& p, void* __restrict__ fb,
                                             double* __restrict__ rho_m,
                                             double* __restrict__ ux_m,
                                             double* __restrict__ uy_m, int x0, int y0,
-                                            const typename Pop<S>::C (*psi_s)[TX + 2],
+                                            const typename Pop<S>::C (*psi_s)[TXN + 2],
                                             typename Pop<S>::C (&f)[RY][9],
                                             const typename Pop<S>::C (&rho)[RY],
                                             const typename Pop<S>::C (&inv)[RY],
@@ -246,8 +246,7 @@ __device__ __forceinline__ void tile_phase2(const DevParams& p, void* __restrict
       psic = psi_s[cy][cx];
     }
     C st[9], ux, uy;
-    collide_node<S, EOS>(p, k, f[r], rho[r], inv[r], d13, d24, d57, d86, psic, C(x), C(y), st,
-                         ux, uy);
+    collide_node<S, EOS>(p, k, f[r], rho[r], inv[r], d13, d24, d57, d86, psic, C(x), C(y), st, ux, uy);
     if constexpr (FIELDS) {
       rho_m[n] = double(rho[r]);
       ux_m[n] = double(ux);
@@ -278,23 +277,25 @@ __device__ __forceinline__ void tile_phase2(const DevParams& p, void* __restrict
 
 
 // One tile (x0, y0) of one lattice: every thread of the CTA calls it with the same arguments.
-// psi_s: shared memory of (TYT RY + 2) x (TX + 2) values.
-template <typename S, int EOS, bool FIELDS, int RY>
+// psi_s: shared memory of (TYN RY + 2) x (TXN + 2) values.
+// PDL: the caller is a kernel of a time step that has not waited for the one before yet; the
+// tile loads its flags first, then waits.
+template <typename S, int EOS, bool FIELDS, int RY, int TYN = TYT, int TXN = TX, bool PDL = false>
 __device__ __forceinline__ void step_tile(const DevParams& p, const void* __restrict__ fa,
                                           void* __restrict__ fb,
                                           const uint8_t* __restrict__ flags,
                                           double* __restrict__ rho_m, double* __restrict__ ux_m,
                                           double* __restrict__ uy_m, int x0, int y0,
-                                          typename Pop<S>::C (*psi_s)[TX + 2]) {
+                                          typename Pop<S>::C (*psi_s)[TXN + 2]) {
   using C = typename StoreTraits<S>::C;
   constexpr bool DEV = StoreTraits<S>::deviation;
-  constexpr int TH = TYT * RY;  // tile height in nodes
+  constexpr int TH = TYN * RY;  // tile height in nodes
 
   const int tx = threadIdx.x, ty = threadIdx.y;
   const int nx = p.nx, ny = p.ny;
   const int N = p.N;  // 9 N < 2^31 (checked at creation): 32-bit element offsets
   // ragged tiles of lattices narrower than a tile wrap more than once
-  const bool small = nx <= TX + 1 || ny <= TH + 1;
+  const bool small = nx <= TXN + 1 || ny <= TH + 1;
   const Consts<C>& k = p.k<C>();
   const C rho_ref = DEV ? k.rho_ref : C(0);
   const C psi_w = k.psi_wall;
@@ -307,13 +308,20 @@ __device__ __forceinline__ void step_tile(const DevParams& p, const void* __rest
   C f[RY][9];
   C rho[RY], inv[RY];
   uint8_t fl[RY];
+  auto own_node = [&](int r) {
+    const int y = y0 + ty + r * TYN;
+    return (y < ny ? y : 0) * nx + xo;
+  };
+  auto load_own_flags = [&] {
+#pragma unroll
+    for (int r = 0; r < RY; ++r)
+      fl[r] = (x <= nx && y0 + ty + r * TYN <= ny) ? flags[LBM_CHK(own_node(r), N)]
+                                                   : uint8_t(FLAG_SOLID);
+  };
   auto load_own = [&] {
 #pragma unroll
     for (int r = 0; r < RY; ++r) {
-      const int y = y0 + ty + r * TYT;
-      const int yo = y < ny ? y : 0;
-      const int n = yo * nx + xo;
-      fl[r] = (x <= nx && y <= ny) ? flags[LBM_CHK(n, N)] : uint8_t(FLAG_SOLID);
+      const int n = own_node(r);
       rho[r] = C(1);
       if (!(fl[r] & FLAG_SOLID)) {
 #pragma unroll
@@ -329,19 +337,19 @@ __device__ __forceinline__ void step_tile(const DevParams& p, const void* __rest
     // kRing threads.  Its loads are issued first, then the own nodes' (the batched FP16 step ran
     // 4.5% faster than with the own loads first), and no psi is computed before both are in
     // flight, so a CTA waits for memory once.
-    constexpr int kRing = 2 * (TX + 2) + 2 * TH;
-    static_assert(kRing <= TX * TYT, "one ring cell per thread");
-    const int c = ty * TX + tx;
-    int hx = 0, hy = 0;
+    constexpr int kRing = 2 * (TXN + 2) + 2 * TH;
+    static_assert(kRing <= TXN * TYN, "one ring cell per thread");
+    const int c = ty * TXN + tx;
+    int hx = 0, hy = 0, ring_node = 0;
     bool ring_fluid = false;
     C v[9];
     if (c < kRing) {
-      if (c < 2 * (TX + 2)) {
-        hx = c < TX + 2 ? c : c - (TX + 2);
-        hy = c < TX + 2 ? 0 : TH + 1;
+      if (c < 2 * (TXN + 2)) {
+        hx = c < TXN + 2 ? c : c - (TXN + 2);
+        hy = c < TXN + 2 ? 0 : TH + 1;
       } else {
-        const int kk = c - 2 * (TX + 2);
-        hx = kk < TH ? 0 : TX + 1;
+        const int kk = c - 2 * (TXN + 2);
+        hx = kk < TH ? 0 : TXN + 1;
         hy = (kk < TH ? kk : kk - TH) + 1;
       }
       int gx = x0 - 1 + hx, gy = y0 - 1 + hy;
@@ -355,29 +363,38 @@ __device__ __forceinline__ void step_tile(const DevParams& p, const void* __rest
       }
       const int m = gy * nx + gx;
       ring_fluid = ring_need && !(flags[LBM_CHK(m, N)] & FLAG_SOLID);
-      if (ring_fluid) {
-#pragma unroll
-        for (int a = 0; a < 9; ++a) v[a] = Pop<S>::load(fa, a, N, m);
-      }
+      ring_node = m;
     }
+    if constexpr (PDL) {
+      load_own_flags();
+      pdl_wait();
+    }
+    if (ring_fluid) {
+#pragma unroll
+      for (int a = 0; a < 9; ++a) v[a] = Pop<S>::load(fa, a, N, ring_node);
+    }
+    if constexpr (!PDL) load_own_flags();
     load_own();
 #pragma unroll
     for (int r = 0; r < RY; ++r) {
       if (!(fl[r] & FLAG_SOLID)) rho[r] = density_of<DEV>(rho_ref, f[r]);
       const C ps = psi_own<C, EOS>(k, rho[r], inv[r]);
-      psi_s[ty + r * TYT + 1][tx + 1] = (fl[r] & FLAG_SOLID) ? psi_w : ps;
+      psi_s[ty + r * TYN + 1][tx + 1] = (fl[r] & FLAG_SOLID) ? psi_w : ps;
     }
     if (c < kRing)
       psi_s[hy][hx] = ring_fluid ? psi_of<C, EOS>(k, density_of<DEV>(rho_ref, v)) : psi_w;
     __syncthreads();
   } else {
+    load_own_flags();
+    if constexpr (PDL) pdl_wait();
     load_own();
 #pragma unroll
     for (int r = 0; r < RY; ++r)
       if (!(fl[r] & FLAG_SOLID)) rho[r] = density_of<DEV>(rho_ref, f[r]);
   }
 
-  tile_phase2<S, EOS, FIELDS, RY>(p, fb, rho_m, ux_m, uy_m, x0, y0, psi_s, f, rho, inv, fl);
+  if constexpr (PDL) pdl_trigger();
+  tile_phase2<S, EOS, FIELDS, RY, TYN, TXN>(p, fb, rho_m, ux_m, uy_m, x0, y0, psi_s, f, rho, inv, fl);
 }
 
 }  // namespace step_core

@@ -418,7 +418,6 @@ __global__ void __launch_bounds__(VW* Vec<S>::VH, Vec<S>::kBlocks)
 
   // ---- own populations and flags ----
   auto load_own = [&] {
-    load_flags<V>(flags, LBM_CHK(n, N - V + 1), fl);
 #pragma unroll
     for (int a = 0; a < 9; ++a) {
       C t[V];
@@ -459,12 +458,16 @@ __global__ void __launch_bounds__(VW* Vec<S>::VH, Vec<S>::kBlocks)
   // 4096^2: FP32 208 us own-first against 217-221 us staged-first; FP16 186-187 us against
   // 198-206 us).
   if constexpr (VT::kOwnFirst) {
+    load_flags<V>(flags, LBM_CHK(n, N - V + 1), fl);
+    pdl_wait();
     load_own();
     stage_copies();
     issue_ring_copies();
   } else {
+    pdl_wait();
     stage_copies();
     issue_ring_copies();
+    load_flags<V>(flags, LBM_CHK(n, N - V + 1), fl);
     load_own();
   }
 
@@ -537,6 +540,7 @@ __global__ void __launch_bounds__(VW* Vec<S>::VH, Vec<S>::kBlocks)
     __syncthreads();  // psi_s complete
   }
 
+  pdl_trigger();
   if (y >= ny) return;  // a wrapped row of a ragged tile: psi only
 
   // ---- collisions of the own nodes ----
@@ -674,18 +678,17 @@ cudaError_t launch_vec_t(const DevParams& p, const void* fa, void* fb, const uin
         pf_flags = make_flags_prefetch_map(&fmap, flags, p.nx, p.ny, TW, VH) ? 1 : 0;
     }
     if (maps) {
-      step_vec_kernel<S, EOS, false, true><<<grid, block, 0, s>>>(
-          p, fa, fb, flags, rho_m, ux_m, uy_m, map, map2, pmap, pmap2, fmap, pf_flags, err);
-      return cudaGetLastError();
+      return launch_pdl(step_vec_kernel<S, EOS, false, true>, grid, block, s, p, fa, fb, flags,
+                        rho_m, ux_m, uy_m, map, map2, pmap, pmap2, fmap, pf_flags, err);
     }
   }
-  if (fields_only)
+  if (fields_only) {
     step_vec_kernel<S, EOS, true, false><<<grid, block, 0, s>>>(
         p, fa, fb, flags, rho_m, ux_m, uy_m, map, map2, pmap, pmap2, fmap, 0, err);
-  else
-    step_vec_kernel<S, EOS, false, false><<<grid, block, 0, s>>>(
-        p, fa, fb, flags, rho_m, ux_m, uy_m, map, map2, pmap, pmap2, fmap, 0, err);
-  return cudaGetLastError();
+    return cudaGetLastError();
+  }
+  return launch_pdl(step_vec_kernel<S, EOS, false, false>, grid, block, s, p, fa, fb, flags, rho_m,
+                    ux_m, uy_m, map, map2, pmap, pmap2, fmap, 0, err);
 }
 
 template <typename S>

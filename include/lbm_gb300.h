@@ -125,7 +125,10 @@ typedef struct {
                         * initial fluid density, set by lbm_init_fields / lbm_init_droplet.     *
                         * Used rounded to the nearest FP32 value                                */
   int32_t kernel_path; /* step kernel, all with the same results bit for bit:                  *
-                        * 0: the fastest measured: for FP32/FP16 deviations with nx % 4 == 0    *
+                        * 0: the fastest measured.  Small and mid-size lattices: scalar tiles   *
+                        *    sized to the lattice that also do the wall pass of the step before  *
+                        *    (the last step's stays a launch of its own; not for Zhao-Yong links *
+                        *    and open channels).  Others, with FP32/FP16 deviations, nx % 4 == 0 *
                         *    and ny >= 8 (FP16: 12) the vectorised kernel (population vectors   *
                         *    of 16 B; the two psi-ring rows of tiles away from the x seam staged *
                         *    by tensor copies (TMA), the rest of the halo by cp.async), otherwise *

@@ -30,7 +30,8 @@ def _nvcc():
 
 
 def _sources():
-    names = CUDA_SOURCES + CXX_SOURCES + ["d2q9.cuh", "step_core.cuh", "tma.cuh", "lbm_internal.h"]
+    names = CUDA_SOURCES + CXX_SOURCES + ["d2q9.cuh", "step_core.cuh", "wall.cuh", "wall_tile.cuh",
+                                           "tma.cuh", "lbm_internal.h"]
     paths = [os.path.join(CSRC, n) for n in names]
     paths.append(os.path.join(os.path.dirname(HERE), "include", "lbm_gb300.h"))
     paths.append(os.path.abspath(__file__))
@@ -58,9 +59,10 @@ def build(force=False, verbose=False, checked=False):
     for src in CUDA_SOURCES:
         obj = os.path.join(objdir, src + ".o")
         # The wall pass is compiled without multiply-add contraction: its per-link arithmetic is
-        # inlined into the single-lattice and the batched kernels, and must round identically in
-        # both so a lattice gives the same bits alone and in a batch.
-        fmad = ["--fmad=false"] if src == "boundary.cu" else []
+        # inlined into the single-lattice and the batched wall kernels and the step kernels, and
+        # must round identically in all of them so a lattice gives the same bits alone and in a
+        # batch.  (The step kernels' own arithmetic is explicitly rounded.)
+        fmad = ["--fmad=false"] if src in ("boundary.cu", "step.cu") else []
         cmd = [nvcc, *ARCH, "-O3", "-lineinfo", "-std=c++17", *fmad, *defs, "-Xcompiler", "-fPIC",
                "-Xcompiler", "-ffp-contract=off", "-c", os.path.join(CSRC, src), "-o", obj]
         procs.append((cmd, subprocess.Popen(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT)))

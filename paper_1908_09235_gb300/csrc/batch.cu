@@ -294,7 +294,7 @@ lbm_status lbm_batch_add(lbm_batch* b, const lbm_domain* d, int64_t steps, int32
     }
   if (free_slot < 0) return LBM_ENOMEM;
   lbm_ctx* c = nullptr;
-  lbm_status st = lbm_create(&d->geometry, &d->eos, d->tau, d->scheme, &b->opt, &c);
+  lbm_status st = create_context(&d->geometry, &d->eos, d->tau, d->scheme, &b->opt, true, &c);
   if (st != LBM_OK) return st;
   c->in_batch = true;
   if (d->init == 1)

@@ -21,22 +21,13 @@
 // formats); each boundary node's mass bookkeeping is FP64 for every format.  (FP64 link
 // arithmetic for the deviation formats was measured: 4.3 us more per step at 4096^2 and 0.25 ms
 // more per batched step of 512 lattices, on GB300's narrow FP64 pipe.)
-#include "d2q9.cuh"
+#include "wall.cuh"
 
 namespace lbm {
 
 namespace {
 
-constexpr uint8_t kFromA = 1;   // X2 is read from lattice A (pre-collision)
-constexpr uint8_t kGhost = 2;   // the link has the ghost-node term chi f_eq(x_s)
-
-// The bracket of Eqs. (8), (20), (22): w_a [1 + 3 e_a.u_s + 4.5 (e_a.u_b)^2 - 1.5 u_b.u_b].
-template <typename T>
-__device__ __forceinline__ T bracket(int a, T usx, T usy, T ubx, T uby) {
-  const T eus = T(ex(a)) * usx + T(ey(a)) * usy;
-  const T eub = T(ex(a)) * ubx + T(ey(a)) * uby;
-  return wgt<T>(a) * (T(1) + T(3) * eus + T(4.5) * eub * eub - T(1.5) * (ubx * ubx + uby * uby));
-}
+using namespace wall;
 
 // One thread per boundary node: the recipe of each of its links.
 __global__ void link_setup_kernel(DevParams p, int nb, const int32_t* __restrict__ bnode,
@@ -154,175 +145,45 @@ __global__ void link_setup_kernel(DevParams p, int nb, const int32_t* __restrict
   }
 }
 
-template <typename S>
-struct Lat {
-  const void* __restrict__ src;  // lattice A: f(t)
-  void* __restrict__ dst;        // lattice B: streamed values of step t
-  int N;
-  double rho_ref;
-};
-
-// Sum over the 8 lanes of a node's group in a fixed tree order (bitwise reproducible); `mask`
-// holds the 8 lanes of the group.
 template <typename T>
-__device__ __forceinline__ T group8_sum(T v, unsigned mask) {
-  v += __shfl_xor_sync(mask, v, 4);
-  v += __shfl_xor_sync(mask, v, 2);
-  v += __shfl_xor_sync(mask, v, 1);
-  return v;
+__global__ void tile_links_kernel(int n_nodes, const TileNode* __restrict__ nodes,
+                                  const int32_t* __restrict__ first,
+                                  const int32_t* __restrict__ boff,
+                                  const uint8_t* __restrict__ ldir, LinkRecipe r,
+                                  const int32_t* __restrict__ local, TileLink<T>* links) {
+  const int k = blockIdx.x * blockDim.x + threadIdx.x;
+  if (k >= n_nodes) return;
+  const TileNode nd = nodes[k];
+  for (int l = boff[nd.b], o = first[k]; l < boff[nd.b + 1]; ++l, ++o) {
+    TileLink<T> q{};
+    q.src = r.src[l];
+    q.x1 = r.x1[l];
+    q.x2 = r.x2[l];
+    q.uf = r.uf[l];
+    q.n = nd.n;
+    q.info = ldir[l] | r.kind[l] << 4 | local[k] << 8;
+    q.c0 = pick<T>(r.c0, r.c0f, l);
+    q.c1 = pick<T>(r.c1, r.c1f, l);
+    q.c2 = pick<T>(r.c2, r.c2f, l);
+    q.chi = pick<T>(r.chi, r.chif, l);
+    q.cus = pick<T>(r.cus, r.cusf, l);
+    links[o] = q;
+  }
 }
 
-template <typename T>
-__device__ __forceinline__ T pick(const double* d, const float* f, int l) {
-  if constexpr (sizeof(T) == 8) return d[l]; else return f[l];
-}
-
-// Boundary node b of a lattice handled by lane k (0..7) of an 8-lane group (node_ok false: a
-// padding group, which still takes part in the shuffles).  Arithmetic type T: FP64 for FP64
-// storage; FP32 for the deviation formats, whose mass bookkeeping is exact instead: each node's
-// imbalance between the stored outgoing and incoming values is summed in FP64 and goes, with the
-// previous step's FP64 rounding residue, into its rest population.  For schemes A and
-// L-Bouzidi + A that is Eq. (18); for B (balanced by construction, Eq. 19) and halfway
-// bounce-back it only returns the FP32 rounding.
+// The wall values written in place, into lattice B and the carry array.
 template <typename S>
-__device__ __forceinline__ void boundary_group(const DevParams& p, int b, int k, bool node_ok,
-                                               const int32_t* __restrict__ bnode,
-                                               const int32_t* __restrict__ boff,
-                                               const uint8_t* __restrict__ ldir,
-                                               const LinkRecipe& r, const Lat<S>& L,
-                                               const double* __restrict__ rho_m,
-                                               const double* __restrict__ ux_m,
-                                               const double* __restrict__ uy_m,
-                                               double* __restrict__ carry,
-                                               double* __restrict__ force, unsigned mask) {
+struct InPlace {
   using T = typename Pop<S>::C;
-  constexpr bool DEV = Pop<S>::dev;
-  const int scheme = p.scheme;
-  const int N = L.N;
-  const bool fix_f0 = scheme == LBM_MOD_A || scheme == LBM_BOUZIDI_L_A;
-  const bool conserving = fix_f0 || scheme == LBM_MOD_B || scheme == LBM_HBB;
-  const bool fict = scheme == LBM_MOD_B || scheme == LBM_BAO;
-  const T rref = DEV ? p.k<T>().rho_ref : T(0);
-  // macro arrays: FP64 for FP64 storage, FP32 (in the same memory) for the deviation formats
-  const T* rhoT = reinterpret_cast<const T*>(rho_m);
-  const T* uxT = reinterpret_cast<const T*>(ux_m);
-  const T* uyT = reinterpret_cast<const T*>(uy_m);
-
-  // first loads: node and link records
-  int n = 0, l0 = 0, nl = 0;
-  if (node_ok) {
-    n = bnode[b];
-    l0 = boff[b];
-    nl = boff[b + 1] - l0;
+  void* f;
+  int N;
+  double* out;
+  __device__ __forceinline__ T incoming(int dst, int a, T v) const {
+    return Pop<S>::store_t(f, dst, N, v);
   }
-  const bool act = node_ok && k < nl;
-  int a = 1, src = 0, dst = 0, x1 = -1, x2 = -1, uf = -1;
-  uint8_t kind = 0;
-  T c0 = T(1), c1 = T(0), c2 = T(0), chi = T(0), cus = T(0);
-  T rho_b = T(1), ubx = T(0), uby = T(0);
-  if (act) {
-    const int l = l0 + k;
-    a = ldir[l];
-    src = r.src[l];
-    dst = r.dst[l];
-    x1 = r.x1[l];
-    x2 = r.x2[l];
-    uf = r.uf[l];
-    kind = r.kind[l];
-    c0 = pick<T>(r.c0, r.c0f, l);
-    c1 = pick<T>(r.c1, r.c1f, l);
-    c2 = pick<T>(r.c2, r.c2f, l);
-    chi = pick<T>(r.chi, r.chif, l);
-    cus = pick<T>(r.cus, r.cusf, l);
-  }
-  // Everything above is fixed for the lattice's lifetime; everything below (the moments in the
-  // macro arrays, the lattice values, the FP64 carry) was written by the kernels before this
-  // one.  Launched as a programmatic dependent of the step kernel, the pass waits here for that
-  // grid to complete and its writes to be visible; otherwise the wait returns at once.
-  pdl_wait();
-  if (act) {
-    rho_b = __ldcg(rhoT + LBM_CHK(n, N));
-    ubx = __ldcg(uxT + n);
-    uby = __ldcg(uyT + n);
-  }
-  // second loads: lattice values (deviations d_ for the FP32 formats; f = d_ + w rho_ref)
-  const T w = wgt<T>(a);
-  const T wr = w * rref;
-  T fo_d = T(0), X1 = T(0), X2 = T(0), usx = T(0), usy = T(0);
-  if (act) {
-    fo_d = Pop<S>::load_t(L.dst, src, N);  // outgoing f*_a(x_b, t)
-    if (x1 >= 0) X1 = Pop<S>::load_t(L.dst, x1, N) + wr;
-    if (x2 >= 0) X2 = Pop<S>::load_t((kind & kFromA) ? L.src : L.dst, x2, N) + wr;
-    if (kind & kGhost) {
-      if (uf >= 0) {
-        usx = __ldcg(uxT + LBM_CHK(uf, N));
-        usy = __ldcg(uyT + uf);
-      } else {
-        usx = cus * ubx;
-        usy = cus * uby;
-      }
-    }
-  }
-  const T fo = fo_d + wr;
-  const bool lane0 = node_ok && k == 0;
-  T f0_d = T(0);
-  if (lane0 && (fix_f0 || (DEV && conserving))) f0_d = Pop<S>::load_t(L.dst, n, N);
-
-  const bool gh = act && (kind & kGhost);
-  const T br = gh ? bracket<T>(a, usx, usy, ubx, uby) : T(0);
-  T rho_s = rho_b;
-  if (fict) {
-    T num = T(0), den = T(0);
-    if (gh) {  // links without a ghost term are halfway bounce-back: chi = 0
-      num = scheme == LBM_MOD_B ? chi * fo : fo;  // Eq. (22) / Eq. (23)
-      den = scheme == LBM_MOD_B ? chi * br : br;
-    }
-    num = group8_sum(num, mask);
-    den = group8_sum(den, mask);
-    if (den != T(0)) rho_s = num / den;
-  }
-  T val = c0 * fo + c1 * X1 + c2 * X2;
-  if (gh) val += chi * ((fict ? rho_s : rho_b) * br);  // Eq. (8) / Eq. (20) in Eq. (7) / (17)
-  T in_d = T(0);
-  if (act) {
-    // a pure bounce-back link (halfway bounce-back or a fallback) copies the stored value
-    const bool copy = DEV && !gh && x1 < 0 && x2 < 0 && c0 == T(1);
-    in_d = Pop<S>::store_t(L.dst, dst, N, copy ? fo_d : val - wr);
-  }
-  if (force) {
-    // Momentum exchange (Sec. 4.2, after Mei et al. 2002): through link a the wall receives
-    // e_a (f*_a(x_b, t) + f_abar(x_b, t+1)), with the incoming value as stored; FP64 sums over
-    // the node's links in the fixed group order, one (fx, fy) per boundary node.
-    const double m = act ? double(fo_d) + double(in_d) + 2.0 * wgt<double>(a) * L.rho_ref : 0.0;
-    const double fx = group8_sum(double(ex(a)) * m, mask);
-    const double fy = group8_sum(double(ey(a)) * m, mask);
-    if (lane0) {
-      force[2 * b] = fx;
-      force[2 * b + 1] = fy;
-    }
-  }
-
-  if constexpr (DEV) {
-    if (conserving) {
-      // exact FP64 imbalance of the stored deviations (the w rho_ref parts cancel)
-      const double dm = group8_sum(act ? double(fo_d) - double(in_d) : 0.0, mask);
-      if (lane0) {
-        const double want = double(f0_d) + dm + __ldcg(carry + b);
-        if (want != double(f0_d)) {
-          const T st = Pop<S>::store_t(L.dst, n, N, T(want));
-          carry[b] = want - double(st);
-        } else {
-          carry[b] = 0.0;
-        }
-      }
-    }
-  } else {
-    if (fix_f0) {
-      const double dm = group8_sum(act ? fo - val : 0.0, mask);  // Eq. (15)
-      if (lane0) Pop<S>::store_t(L.dst, n, N, f0_d + dm);     // Eq. (18)
-    }
-  }
-}
+  __device__ __forceinline__ T rest(int n, T v) const { return Pop<S>::store_t(f, n, N, v); }
+  __device__ __forceinline__ void carry(int b, double c) const { out[b] = c; }
+};
 
 // Channel ends (Sec. 4.2), after streaming and the wall pass; one thread per row j.  Inlet
 // i = 0: the populations entering from the left (1, 5, 8) follow from the prescribed velocity
@@ -366,22 +227,25 @@ __global__ void __launch_bounds__(128) boundary_kernel(DevParams p, int nb,
                                                        const int32_t* __restrict__ bnode,
                                                        const int32_t* __restrict__ boff,
                                                        const uint8_t* __restrict__ ldir,
-                                                       LinkRecipe r, Lat<S> L,
-                                                       const double* __restrict__ rho_m,
-                                                       const double* __restrict__ ux_m,
-                                                       const double* __restrict__ uy_m,
-                                                       double* __restrict__ carry,
+                                                       LinkRecipe r, const void* fa, void* fb,
+                                                       const double* rho_m, const double* ux_m,
+                                                       const double* uy_m, const double* carry_in,
+                                                       double* carry_out,
                                                        double* __restrict__ force, int wall_ctas,
                                                        const uint8_t* __restrict__ flags,
                                                        double u_in) {
   if ((int)blockIdx.x >= wall_ctas) {
-    open_row<S>(p, (blockIdx.x - wall_ctas) * blockDim.x + threadIdx.x, L.dst, flags, u_in);
+    open_row<S>(p, (blockIdx.x - wall_ctas) * blockDim.x + threadIdx.x, fb, flags, u_in);
     return;
   }
   const int gt = blockIdx.x * blockDim.x + threadIdx.x;
-  const int b = gt >> 3;
-  boundary_group<S>(p, b, gt & 7, b < nb, bnode, boff, ldir, r, L, rho_m, ux_m, uy_m, carry,
-                    force, 0xffffffffu);
+  const int b = gt >> 3, k = gt & 7;
+  const auto q = load_link<typename Pop<S>::C>(b, k, b < nb, bnode, boff, ldir, r);
+  // the link records are fixed for the lattice's lifetime; everything read below was written by
+  // the kernels before this one
+  pdl_wait();
+  wall_values<S>(p, b, k, b < nb, q, Lat<S>{fa, fb, p.N, p.rho_ref}, rho_m, ux_m, uy_m, carry_in,
+                 InPlace<S>{fb, p.N, carry_out}, force, 0xffffffffu);
 }
 
 template <typename S>
@@ -408,9 +272,10 @@ __global__ void __launch_bounds__(128, 12) batch_boundary_kernel(const BatchDoma
     const BatchDomain& D = doms[it.x];
     if (D.steps_left <= 0) continue;  // uniform over the group
     const int cur = D.cur;
-    const Lat<S> L{D.f[cur], D.f[cur ^ 1], D.p.N, D.p.rho_ref};
-    boundary_group<S>(D.p, it.y, k, true, D.bnode, D.boff, D.ldir, D.recipe, L, D.rho_m, D.ux_m,
-                      D.uy_m, D.carry, nullptr, mask);
+    const auto q = load_link<typename Pop<S>::C>(it.y, k, true, D.bnode, D.boff, D.ldir, D.recipe);
+    wall_values<S>(D.p, it.y, k, true, q, Lat<S>{D.f[cur], D.f[cur ^ 1], D.p.N, D.p.rho_ref},
+                   D.rho_m, D.ux_m, D.uy_m, D.carry, InPlace<S>{D.f[cur ^ 1], D.p.N, D.carry},
+                   nullptr, mask);
   }
 }
 
@@ -431,15 +296,16 @@ unsigned wall_threads(long long threads) { return threads <= 32LL * 152 * 4 ? 32
 template <typename S>
 cudaError_t launch_b(const DevParams& p, int nb, const int32_t* bnode, const int32_t* boff,
                      const uint8_t* ldir, LinkRecipe r, const void* fa, void* fb,
-                     const double* rho_m, const double* ux_m, const double* uy_m, double* carry,
-                     double* force, const uint8_t* open_flags, double u_in, cudaStream_t s) {
-  Lat<S> L{fa, fb, p.N, p.rho_ref};  // rho_ref also in p.k<T>() for the FP32 formats
+                     const double* rho_m, const double* ux_m, const double* uy_m,
+                     const double* carry_in, double* carry_out, double* force,
+                     const uint8_t* open_flags, double u_in, cudaStream_t s) {
   const long long threads = 8LL * nb;
   const unsigned nt = wall_threads(threads + (open_flags ? p.ny : 0));
   const unsigned wall = (unsigned)((threads + nt - 1) / nt);
   const unsigned ends = open_flags ? (p.ny + nt - 1) / nt : 0;
   return launch_pdl(boundary_kernel<S>, dim3(wall + ends), dim3(nt), s, p, nb, bnode, boff, ldir,
-                    r, L, rho_m, ux_m, uy_m, carry, force, (int)wall, open_flags, u_in);
+                    r, fa, fb, rho_m, ux_m, uy_m, carry_in, carry_out, force, (int)wall, open_flags,
+                    u_in);
 }
 
 size_t align256(size_t v) { return (v + 255) / 256 * 256; }
@@ -483,6 +349,23 @@ cudaError_t launch_link_setup(const DevParams& p, int nb, const int32_t* bnode,
   return cudaGetLastError();
 }
 
+size_t tile_link_bytes(int precision) {
+  return precision == LBM_FP64 ? sizeof(TileLink<double>) : sizeof(TileLink<float>);
+}
+
+cudaError_t launch_tile_links(int precision, int n_nodes, const TileNode* nodes,
+                              const int32_t* first, const int32_t* local, const int32_t* boff,
+                              const uint8_t* ldir, LinkRecipe r, void* links, cudaStream_t s) {
+  const int grid = (n_nodes + 127) / 128;
+  if (precision == LBM_FP64)
+    tile_links_kernel<double><<<grid, 128, 0, s>>>(n_nodes, nodes, first, boff, ldir, r, local,
+                                                   (TileLink<double>*)links);
+  else
+    tile_links_kernel<float><<<grid, 128, 0, s>>>(n_nodes, nodes, first, boff, ldir, r, local,
+                                                  (TileLink<float>*)links);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_batch_boundary(int precision, const BatchDomain* doms, const int2* items,
                                   const int* n_items, int grid, cudaStream_t s) {
   if (precision == LBM_FP32_DEV)
@@ -519,16 +402,16 @@ cudaError_t launch_batch_advance(BatchDomain* doms, int n_doms, int* claim, cuda
 cudaError_t launch_boundary(int precision, const DevParams& p, int nb, const int32_t* bnode,
                             const int32_t* boff, const uint8_t* ldir, LinkRecipe r,
                             const void* fa, void* fb, const double* rho_m, const double* ux_m,
-                            const double* uy_m, double* carry, double* force,
-                            const uint8_t* open_flags, double u_in, cudaStream_t s) {
+                            const double* uy_m, const double* carry_in, double* carry_out,
+                            double* force, const uint8_t* open_flags, double u_in, cudaStream_t s) {
   if (nb <= 0) return cudaSuccess;
   if (precision == LBM_FP32_DEV)
-    return launch_b<float>(p, nb, bnode, boff, ldir, r, fa, fb, rho_m, ux_m, uy_m, carry, force,
+    return launch_b<float>(p, nb, bnode, boff, ldir, r, fa, fb, rho_m, ux_m, uy_m, carry_in, carry_out, force,
                            open_flags, u_in, s);
   if (precision == LBM_FP16_DEV)
-    return launch_b<__half>(p, nb, bnode, boff, ldir, r, fa, fb, rho_m, ux_m, uy_m, carry, force,
+    return launch_b<__half>(p, nb, bnode, boff, ldir, r, fa, fb, rho_m, ux_m, uy_m, carry_in, carry_out, force,
                             open_flags, u_in, s);
-  return launch_b<double>(p, nb, bnode, boff, ldir, r, fa, fb, rho_m, ux_m, uy_m, carry, force,
+  return launch_b<double>(p, nb, bnode, boff, ldir, r, fa, fb, rho_m, ux_m, uy_m, carry_in, carry_out, force,
                           open_flags, u_in, s);
 }
 

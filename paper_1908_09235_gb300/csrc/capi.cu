@@ -87,13 +87,15 @@ cudaError_t launch_bulk(lbm_ctx* c, cudaStream_t s, int cur) {
                      c->uy_m, false, s, c->kernel_path, c->err_flag);
 }
 
-// The wall pass and, in channel mode, the channel ends of a step from lattice cur.
-lbm_status launch_walls(lbm_ctx* c, cudaStream_t s, int cur) {
+// The wall pass and, in channel mode, the channel ends of a step from lattice cur; m: which set of
+// moments the step stored and which set of residues is current.  The new residues go to set 0.
+lbm_status launch_walls(lbm_ctx* c, cudaStream_t s, int cur, int m = 0) {
   void* fb = c->f[1 - cur];
   const bool together = c->open_x && c->ends_with_wall && c->nb > 0;
   cudaError_t e = launch_boundary(c->precision, c->p, (int)c->nb, c->bnode, c->boff, c->ldir,
-                                  c->recipe, c->f[cur], fb, c->rho_m, c->ux_m, c->uy_m, c->carry,
-                                  c->track_force ? c->force : nullptr,
+                                  c->recipe, c->f[cur], fb, m ? c->macro2[0] : c->rho_m,
+                                  m ? c->macro2[1] : c->ux_m, m ? c->macro2[2] : c->uy_m,
+                                  m ? c->carry2 : c->carry, c->carry, c->track_force ? c->force : nullptr,
                                   together ? c->flags : nullptr, c->u_in, s);
   if (e != cudaSuccess) return cuda_fail(c, e, "boundary kernel launch");
   if (c->open_x && !together) {
@@ -109,15 +111,44 @@ lbm_status launch_one_step(lbm_ctx* c, cudaStream_t s, int cur) {
   return launch_walls(c, s, cur);
 }
 
+// The wall pass of a step can be done by the next step's kernel (Zhao-Yong's reads the lattice that
+// kernel overwrites; the channel ends come after the wall pass).
+bool walls_in_steps(const lbm_ctx* c) {
+  return c->tiles_shape >= 0 && c->nb > 0 && !c->open_x && c->p.scheme != LBM_ZHAO_YONG;
+}
+
+// n steps from lattice cur, launched one after the other.  Where walls_in_steps, every kernel but
+// the first applies the wall pass of the step before it and only the last step's is a launch of its
+// own, so the lattice is complete between calls; the moments and residues a kernel reads were
+// stored in one set by the step before, its own go to the other.
+lbm_status launch_steps(lbm_ctx* c, cudaStream_t s, int cur, int n) {
+  lbm_status st = LBM_OK;
+  if (!walls_in_steps(c)) {
+    for (int k = 0; k < n && st == LBM_OK; ++k, cur = 1 - cur) st = launch_one_step(c, s, cur);
+    return st;
+  }
+  double* macro[2][3] = {{c->rho_m, c->ux_m, c->uy_m}, {c->macro2[0], c->macro2[1], c->macro2[2]}};
+  double* carry[2] = {c->carry, c->carry2};
+  for (int k = 0; k < n; ++k, cur = 1 - cur) {
+    const int m = k & 1;
+    WallIn wi = c->tiles;
+    wi.rho = macro[1 - m][0];
+    wi.ux = macro[1 - m][1];
+    wi.uy = macro[1 - m][2];
+    wi.carry_in = carry[1 - m];
+    wi.carry_out = carry[m];
+    const cudaError_t e =
+        launch_step_tiles(c->tiles_shape, c->precision, c->p, c->f[cur], c->f[1 - cur], c->flags,
+                          macro[m][0], macro[m][1], macro[m][2], k > 0 ? &wi : nullptr, s);
+    if (e != cudaSuccess) return cuda_fail(c, e, "step kernel launch");
+  }
+  return n > 0 ? launch_walls(c, s, 1 - cur, (n - 1) & 1) : LBM_OK;
+}
+
 lbm_status build_graph(lbm_ctx* c, int parity) {
   cudaGraph_t graph = nullptr;
   LBM_CUDA(c, cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeThreadLocal));
-  int cur = parity;
-  lbm_status st = LBM_OK;
-  for (int k = 0; k < c->graph_steps && st == LBM_OK; ++k) {
-    st = launch_one_step(c, c->cap_stream, cur);
-    cur = 1 - cur;
-  }
+  const lbm_status st = launch_steps(c, c->cap_stream, parity, c->graph_steps);
   cudaError_t e = cudaStreamEndCapture(c->cap_stream, &graph);
   if (st != LBM_OK) {
     if (graph) cudaGraphDestroy(graph);
@@ -175,6 +206,99 @@ lbm_status lbm_coexistence(const lbm_eos* eos, double* rho_l, double* rho_v) {
 
 lbm_status lbm_create(const lbm_geometry* geo, const lbm_eos* eos, double tau, int32_t scheme,
                       const lbm_options* opt, lbm_ctx** out) {
+  return create_context(geo, eos, tau, scheme, opt, false, out);
+}
+
+}  // extern "C"
+
+namespace {
+
+// Cells of a tile of the given width (size) and its ring that hold position i of a periodic axis
+// of n nodes: up to three (tile, cell, owned), cell 0 and width + 1 being the ring.
+struct AxisCells {
+  int count = 0;
+  int tile[3], cell[3];
+  bool owned[3];
+  void add(int t, int c, bool o) {
+    tile[count] = t;
+    cell[count] = c;
+    owned[count++] = o;
+  }
+  AxisCells(int i, int n, int size) {
+    const int t = i / size, last = (n - 1) / size;
+    add(t, i - t * size + 1, true);
+    if (i % size == 0 && t > 0) add(t - 1, size + 1, false);         // right ring of the tile before
+    if (i % size == size - 1 && t < last) add(t + 1, 0, false);      // left ring of the tile after
+    if (i == 0) add(last, n - last * size + 1, false);               // past the last column
+    if (i == n - 1) add(0, 0, false);                                // before the first column
+  }
+};
+
+// The tables of WallIn on the host: from the boundary list (nodes bnode, their link offsets boff and
+// directions ldir), for tiles of tw x th nodes, with the nodes of their rings (ring) or without.
+struct TileTables {
+  std::vector<int4> heads;
+  std::vector<TileNode> nodes;
+  std::vector<int32_t> first, local;  // per node: its first link in the table, its place in the tile
+  int links = 0, max_links = 0, max_nodes = 0;
+
+  TileTables(int nb, const int32_t* bnode, const int32_t* boff, const uint8_t* ldir, int nx,
+             int ny, int tw, int th, bool ring) {
+    const int tx = (nx + tw - 1) / tw, ty = (ny + th - 1) / th;
+    std::vector<std::pair<int, TileNode>> all;
+    all.reserve(2 * (size_t)nb);
+    for (int b = 0; b < nb; ++b) {
+      const int n = bnode[b];
+      int mask = 0;  // the directions opposite to the cut ones
+      for (int l = boff[b]; l < boff[b + 1]; ++l) mask |= 1 << (((ldir[l] - 1) ^ 2) + 1);
+      const AxisCells cx(n % nx, nx, tw), cy(n / nx, ny, th);
+      for (int v = 0; v < cy.count; ++v)
+        for (int u = 0; u < cx.count; ++u) {
+          const bool owned = cx.owned[u] && cy.owned[v];
+          if (owned || ring)
+            all.emplace_back(cy.tile[v] * tx + cx.tile[u],
+                             TileNode{n, b, (cy.cell[v] * (tw + 2) + cx.cell[u]) |
+                                                mask << kMaskShift | (owned ? kOwnedNode : 0),
+                                      boff[b + 1] - boff[b]});
+        }
+    }
+    heads.assign((size_t)tx * ty, int4{0, 0, 0, 0});
+    for (const auto& e : all) {
+      heads[e.first].y += e.second.links;
+      ++heads[e.first].w;
+    }
+    int at = 0;
+    for (auto& h : heads) {
+      h.x = links;
+      h.z = at;
+      links += h.y;
+      at += h.w;
+      max_links = h.y > max_links ? h.y : max_links;
+      max_nodes = h.w > max_nodes ? h.w : max_nodes;
+      h.y = h.w = 0;  // counted again below
+    }
+    nodes.resize(all.size());
+    first.resize(all.size());
+    local.resize(all.size());
+    for (const auto& e : all) {
+      int4& h = heads[e.first];
+      TileNode nd = e.second;
+      const int count = nd.links, k = h.z + h.w;
+      nd.links = h.y << 8 | count;
+      nodes[k] = nd;
+      first[k] = h.x + h.y;
+      local[k] = h.w;
+      h.y += count;
+      ++h.w;
+    }
+  }
+};
+
+}  // namespace
+
+lbm_status lbm::create_context(const lbm_geometry* geo, const lbm_eos* eos, double tau,
+                               int32_t scheme, const lbm_options* opt, bool in_batch,
+                               lbm_ctx** out) {
   if (!out) return LBM_EINVAL;
   *out = nullptr;
   if (!geo || !eos) return LBM_EINVAL;
@@ -361,15 +485,83 @@ lbm_status lbm_create(const lbm_geometry* geo, const lbm_eos* eos, double tau, i
                                c->recipe, c->stream)) != cudaSuccess)
       return bail(e, "link setup");
   }
-  // fluid node count (host, once)
-  std::vector<uint8_t> hf(N);
+  // fluid node count (host, once), and the boundary list for the tables of the step kernels that do
+  // the wall pass themselves
+  int tw = 0, th = 0;
+  const int shape = in_batch || c->nb == 0 || (opt && opt->kernel_path != 0)
+                        ? -1
+                        : pick_step_tiles(precision, eos->kind, geo->nx, geo->ny, &tw, &th);
+  std::vector<uint8_t> hf(N), h_ldir;
+  std::vector<int32_t> h_bnode, h_boff;
   if ((e = cudaMemcpyAsync(hf.data(), c->flags, N, cudaMemcpyDeviceToHost, c->stream)) !=
       cudaSuccess)
     return bail(e, "copy flags");
+  if (shape >= 0) {
+    h_bnode.resize(c->nb);
+    h_boff.resize(c->nb + 1);
+    h_ldir.resize(c->nl);
+    if ((e = cudaMemcpyAsync(h_bnode.data(), c->bnode, c->nb * 4, cudaMemcpyDeviceToHost,
+                             c->stream)) != cudaSuccess ||
+        (e = cudaMemcpyAsync(h_boff.data(), c->boff, (c->nb + 1) * 4, cudaMemcpyDeviceToHost,
+                             c->stream)) != cudaSuccess ||
+        (e = cudaMemcpyAsync(h_ldir.data(), c->ldir, c->nl, cudaMemcpyDeviceToHost,
+                             c->stream)) != cudaSuccess)
+      return bail(e, "copy links");
+  }
   if ((e = cudaStreamSynchronize(c->stream)) != cudaSuccess) return bail(e, "sync");
   long long nf = 0;
   for (size_t k = 0; k < N; ++k) nf += (hf[k] & FLAG_SOLID) ? 0 : 1;
   c->n_fluid = nf;
+
+  // ---- third allocation: the wall pass within the step kernels ----
+  if (shape >= 0) {
+    const TileTables tt((int)c->nb, h_bnode.data(), h_boff.data(), h_ldir.data(), geo->nx, geo->ny,
+                        tw, th, eos->kind != LBM_EOS_NONE);
+    // the tile's tables in shared memory (beside psi, within the 48 KB of a plain launch); a geometry
+    // with more walls in a tile than that keeps the wall pass apart
+    const size_t smem = 16u * tt.max_links + 10 * 8 * (size_t)tt.max_nodes + 4 * (tw + 2) * (th + 2);
+    const bool fits = smem + 64 <= 40 * 1024;
+    const size_t nn = tt.nodes.size(), nm = precision == LBM_FP64 ? 3 * align_up(N * 8) : 0;
+    const size_t tables = align_up(tt.heads.size() * sizeof(int4)) +
+                          align_up(nn * sizeof(TileNode)) + 2 * align_up(nn * 4);
+    void* base3 = dev_alloc(c, tables + align_up(tt.links * tile_link_bytes(precision)) +
+                                   align_up(c->nb * 8) + nm);
+    if (!base3) {
+      release_all(c);
+      delete c;
+      return LBM_ENOMEM;
+    }
+    Carver c3{(char*)base3};
+    int4* heads = c3.take<int4>(tt.heads.size());
+    TileNode* nodes = c3.take<TileNode>(nn);
+    int32_t* first = c3.take<int32_t>(nn);
+    int32_t* local = c3.take<int32_t>(nn);
+    void* links = c3.take<char>(tt.links * tile_link_bytes(precision));
+    c->carry2 = c3.take<double>(c->nb);
+    // the deviation formats store FP32 moments: the second set fits behind the first
+    double* set0[3] = {c->rho_m, c->ux_m, c->uy_m};
+    for (int k = 0; k < 3; ++k)
+      c->macro2[k] = precision == LBM_FP64 ? c3.take<double>(N)
+                                           : reinterpret_cast<double*>((float*)set0[k] + N);
+    std::vector<char> up(tables);  // one upload
+    auto at = [&](const void* dev) { return up.data() + ((const char*)dev - (char*)base3); };
+    std::memcpy(at(heads), tt.heads.data(), tt.heads.size() * sizeof(int4));
+    std::memcpy(at(nodes), tt.nodes.data(), nn * sizeof(TileNode));
+    std::memcpy(at(first), tt.first.data(), nn * 4);
+    std::memcpy(at(local), tt.local.data(), nn * 4);
+    e = cudaMemcpyAsync(base3, up.data(), tables, cudaMemcpyHostToDevice, c->stream);
+    if (e == cudaSuccess)
+      e = launch_tile_links(precision, (int)nn, nodes, first, local, c->boff, c->ldir, c->recipe,
+                            links, c->stream);
+    if (e != cudaSuccess) return bail(e, "tile tables");
+    c->tiles.heads = heads;
+    c->tiles.nodes = nodes;
+    c->tiles.links = links;
+    c->tiles.max_links = tt.max_links;
+    c->tiles.max_nodes = tt.max_nodes;
+    c->tiles.cells = (tw + 2) * (th + 2);
+    c->tiles_shape = fits ? shape : -1;
+  }
   if ((e = cudaMemsetAsync(c->f[0], 0, c->lattice_bytes, c->stream)) != cudaSuccess)
     return bail(e, "memset f0");
   if ((e = cudaMemsetAsync(c->f[1], 0, c->lattice_bytes, c->stream)) != cudaSuccess)
@@ -383,6 +575,8 @@ lbm_status lbm_create(const lbm_geometry* geo, const lbm_eos* eos, double tau, i
   *out = c;
   return LBM_OK;
 }
+
+extern "C" {
 
 void lbm_destroy(lbm_ctx* c) {
   if (!c) return;
@@ -464,12 +658,10 @@ lbm_status lbm_step(lbm_ctx* c, int32_t n) {
     n -= c->graph_steps;
     c->steps += c->graph_steps;  // even: parity unchanged
   }
-  for (; n > 0; --n) {
-    lbm_status st = launch_one_step(c, c->stream, c->cur);
-    if (st != LBM_OK) return st;
-    c->cur = 1 - c->cur;
-    ++c->steps;
-  }
+  const lbm_status st = launch_steps(c, c->stream, c->cur, n);
+  if (st != LBM_OK) return st;
+  c->cur ^= n & 1;
+  c->steps += n;
   return LBM_OK;
 }
 

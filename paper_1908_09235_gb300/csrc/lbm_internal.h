@@ -70,6 +70,7 @@ struct GeomParams {
 };
 
 struct LinkRecipe;
+struct WallIn;
 
 // ---- launchers (implemented in the .cu files) ----
 // geometry.cu
@@ -103,6 +104,14 @@ cudaError_t launch_step(int precision, const DevParams& p, const void* fa, void*
                         const uint8_t* flags, double* rho_m, double* ux_m, double* uy_m,
                         bool fields_only, cudaStream_t s, int path = 0, int* err = nullptr);
 
+// The scalar tiles in the shapes of small lattices, whose step kernels can apply the previous
+// step's wall pass themselves (wi; nullptr: a plain step).  pick_step_tiles: the shape for a
+// lattice and its tile size, or -1 where the wall pass is a launch of its own.
+int pick_step_tiles(int precision, int eos, int nx, int ny, int* tw, int* th);
+cudaError_t launch_step_tiles(int shape, int precision, const DevParams& p, const void* fa,
+                              void* fb, const uint8_t* flags, double* rho_m, double* ux_m,
+                              double* uy_m, const WallIn* wi, cudaStream_t s);
+
 // boundary.cu
 // Per-link recipe of the wall pass, fixed at creation (depends on q, tau and the scheme only):
 //   f_abar(x_b, t+1) = c0 fo + c1 X1 + c2 X2 + chi rho' w_a [1 + 3 e.u_s + 4.5 (e.u_b)^2 - 1.5 u_b^2]
@@ -126,6 +135,33 @@ struct LinkRecipe {
   float* chif;
   float* cusf;
 };
+// What a step kernel needs to apply the previous step's wall pass to its source lattice while it
+// loads it (csrc/wall_tile.cuh), instead of a separate pass over that lattice.
+// A link of a tile, its recipe gathered in one record: info is its direction | kind << 4 | its node
+// in the tile << 8.
+template <typename T>
+struct alignas(16) TileLink {
+  int32_t src, x1, x2, uf, n, info;
+  T c0, c1, c2, chi, cus, pad;
+};
+// A boundary node of a tile: n its index in the lattice, b in the boundary list; cell: the cell
+// cy (w + 2) + cx in the tile (w nodes wide) with its ring | the directions that hold a wall value
+// << kMaskShift | kOwnedNode where the tile owns the node; links: first link in the tile << 8 | count.
+struct alignas(16) TileNode {
+  int32_t n, b, cell, links;
+};
+constexpr int kCellMask = 0xfff, kMaskShift = 12, kOwnedNode = 1 << 24;
+struct WallIn {
+  const int4* heads;  // per tile: first link, links, first node, nodes
+  const void* links;  // TileLink<T>
+  const TileNode* nodes;
+  int max_links, max_nodes;  // of a tile
+  int cells;                 // (w + 2) (h + 2) of a tile
+  const double *rho, *ux, *uy;  // the moments that the step before stored
+  const double* carry_in;       // the FP64 residues before and after
+  double* carry_out;
+};
+
 // One lattice of a batch as the batched kernels see it.  cur and steps_left are advanced on
 // the device after every step (batch_advance_kernel), so a captured graph stays valid while
 // lattices join and leave the batch.
@@ -153,13 +189,20 @@ cudaError_t launch_link_setup(const DevParams& p, int nb, const int32_t* bnode,
 cudaError_t launch_boundary(int precision, const DevParams& p, int nb, const int32_t* bnode,
                             const int32_t* boff, const uint8_t* ldir, LinkRecipe r,
                             const void* fa, void* fb, const double* rho_m, const double* ux_m,
-                            const double* uy_m, double* carry, double* force,
-                            const uint8_t* open_flags, double u_in, cudaStream_t s);
+                            const double* uy_m, const double* carry_in, double* carry_out,
+                            double* force, const uint8_t* open_flags, double u_in, cudaStream_t s);
 // open_flags (with nb > 0): the node flags, to do the channel ends in the same launch (only where
 // they and the wall pass touch different nodes), or nullptr.  force: per boundary node (fx, fy) of the momentum exchange with the walls, or nullptr
 // Channel ends (velocity inlet at column 0, fully developed outlet at column nx - 1)
 cudaError_t launch_open_x(int precision, const DevParams& p, void* fb, const uint8_t* flags,
                           double u_in, cudaStream_t s);
+
+// The link records of tiles: node k of the table, node local[k] of its tile, has its links from
+// first[k] on.
+cudaError_t launch_tile_links(int precision, int n_nodes, const TileNode* nodes,
+                              const int32_t* first, const int32_t* local, const int32_t* boff, const uint8_t* ldir,
+                              LinkRecipe r, void* links, cudaStream_t s);
+size_t tile_link_bytes(int precision);
 
 // batched kernels (step.cu, boundary.cu, batch.cu)
 int batch_tile_rows(int ry);
@@ -210,6 +253,11 @@ cudaError_t launch_step_tma(const void* map, const void* flag_map, const DevPara
 constexpr int kErrUnstable = 1;  // bits of the context's device error word
 constexpr int kErrTimeout = 4;
 
+// capi.cu
+// lbm_create; in_batch: the lattice will be stepped by a batch's kernels only.
+lbm_status create_context(const lbm_geometry* geo, const lbm_eos* eos, double tau, int32_t scheme,
+                          const lbm_options* opt, bool in_batch, lbm_ctx** out);
+
 // eos_host.cpp
 bool cs_critical_point(double a, double b, double R, double* Tc, double* rhoc);
 bool cs_maxwell(double a, double b, double R, double T, double* rho_l, double* rho_v);
@@ -239,6 +287,12 @@ struct lbm_ctx {
   uint8_t* ldir = nullptr;
   double* lq = nullptr;
   double* carry = nullptr;
+  // the wall pass within the step kernel (WallIn): shape of launch_step_tiles or -1, the tables,
+  // and the second set of moments and residues that alternate with the first from step to step
+  int tiles_shape = -1;
+  lbm::WallIn tiles{};
+  double* macro2[3] = {nullptr, nullptr, nullptr};
+  double* carry2 = nullptr;
   double* force = nullptr;    // per boundary node (fx, fy) of the last step's momentum exchange
   bool track_force = false;   // the wall pass fills `force` (lbm_options.track_force, inflow)
   bool open_x = false;        // channel mode (lbm_set_inflow)

@@ -10,7 +10,8 @@
 // A CTA covers a 32 x (8 RY) tile; each thread keeps the 9 populations of its RY nodes in
 // registers.  psi of the tile and of a one-node ring around it goes to shared memory (ring nodes
 // recompute their density from their own 9 populations), so the force needs no second pass over
-// memory.  RY = 4 rows per thread for FP32 arithmetic, 2 for FP64 (register budget).
+// memory.  RY = 4 rows per thread for FP32 arithmetic, 2 for FP64 (register budget).  Lattices that
+// do not fill the GPU so take smaller tiles (pick_step_tiles).
 #include "step_core.cuh"
 
 namespace lbm {
@@ -37,6 +38,23 @@ __global__ void __launch_bounds__(TXN* TYN, tile_ctas<S, RY>() * (TX * TYT) / (T
   __shared__ C psi_s[TYN * RY + 2][TXN + 2];
   step_tile<S, EOS, FIELDS, RY, TYN, TXN, true>(p, fa, fb, flags, rho_m, ux_m, uy_m,
                                                 blockIdx.x * TXN, blockIdx.y * TYN * RY, psi_s);
+}
+
+// The same tile, whose source lattice has not had its wall pass yet (WallIn).  MODE: step_tile's WALL;
+// 1 may use 128 registers (the CTAs of a small lattice do not fill the SMs anyway).
+template <typename S, int EOS, int TXN, int TYN, int RY, int MODE>
+__global__ void __launch_bounds__(TXN* TYN,
+                                  (MODE == 1 ? 2 : tile_ctas<S, RY>()) * (TX * TYT) / (TXN * TYN))
+    step_wall_kernel(const __grid_constant__ DevParams p, const void* __restrict__ fa,
+                     void* __restrict__ fb, const uint8_t* __restrict__ flags,
+                     double* __restrict__ rho_m, double* __restrict__ ux_m,
+                     double* __restrict__ uy_m, const __grid_constant__ WallIn wi) {
+  using C = typename StoreTraits<S>::C;
+  __shared__ C psi_s[TYN * RY + 2][TXN + 2];
+  extern __shared__ __align__(16) unsigned char wall_smem[];
+  step_tile<S, EOS, false, RY, TYN, TXN, true, MODE>(
+      p, fa, fb, flags, rho_m, ux_m, uy_m, blockIdx.x * TXN, blockIdx.y * TYN * RY, psi_s, &wi,
+      blockIdx.y * gridDim.x + blockIdx.x, wall_smem);
 }
 
 // Many lattices in one launch: a persistent grid works through a queue of tiles (domain, x0,
@@ -94,8 +112,9 @@ template <typename S, int EOS>
 cudaError_t launch_t(const DevParams& p, const void* fa, void* fb, const uint8_t* flags,
                      double* rho_m, double* ux_m, double* uy_m, bool fields_only,
                      cudaStream_t s) {
-  return launch_shape<S, EOS, TX, TYT, StoreTraits<S>::RY>(p, fa, fb, flags, rho_m, ux_m, uy_m,
-                                                          fields_only, s);
+  // (FP64 without psi has no ring to share: one row a thread, 2048^2 525 against 545 us)
+  constexpr int RY = sizeof(S) == 8 && EOS == LBM_EOS_NONE ? 1 : StoreTraits<S>::RY;
+  return launch_shape<S, EOS, TX, TYT, RY>(p, fa, fb, flags, rho_m, ux_m, uy_m, fields_only, s);
 }
 
 template <typename S>
@@ -109,6 +128,59 @@ cudaError_t launch_s(const DevParams& p, const void* fa, void* fb, const uint8_t
       return launch_t<S, LBM_EOS_CS>(p, fa, fb, flags, rho_m, ux_m, uy_m, fields_only, s);
     default:
       return launch_t<S, LBM_EOS_NONE>(p, fa, fb, flags, rho_m, ux_m, uy_m, fields_only, s);
+  }
+}
+
+template <typename S, int EOS, int TXN, int TYN, int RY, int MODE>
+cudaError_t launch_wall_shape(const DevParams& p, const void* fa, void* fb, const uint8_t* flags,
+                              double* rho_m, double* ux_m, double* uy_m, const WallIn* wi,
+                              cudaStream_t s) {
+  constexpr int TH = TYN * RY;
+  const dim3 block(TXN, TYN), grid((p.nx + TXN - 1) / TXN, (p.ny + TH - 1) / TH);
+  if (!wi)
+    return launch_pdl(step_kernel<S, EOS, false, TXN, TYN, RY>, grid, block, s, p, fa, fb, flags,
+                      rho_m, ux_m, uy_m);
+  const size_t smem = wall::tile_wall_bytes<typename Pop<S>::C>(wi->max_links, wi->max_nodes,
+                                                                (TXN + 2) * (TH + 2));
+  return launch_pdl_smem(step_wall_kernel<S, EOS, TXN, TYN, RY, MODE>, grid, block, smem, s, p, fa, fb,
+                         flags, rho_m, ux_m, uy_m, *wi);
+}
+
+struct TileShape {
+  int w, ty, ry, mode;  // threads in x and y, rows per thread, step_tile's WALL
+};
+constexpr TileShape kShapes[] = {{16, 4, 1, 1}, {16, 8, 1, 1}, {32, 8, 1, 1},
+                                 {32, 8, 1, 2}, {32, 8, 2, 2}, {32, 8, 4, 2}};
+
+template <typename S, int EOS>
+cudaError_t launch_tiles_t(int shape, const DevParams& p, const void* fa, void* fb,
+                           const uint8_t* flags, double* rho_m, double* ux_m, double* uy_m,
+                           const WallIn* wi, cudaStream_t s) {
+#define LBM_SHAPE(k)                                                                         \
+  if (shape == k)                                                                            \
+  return launch_wall_shape<S, EOS, kShapes[k].w, kShapes[k].ty, kShapes[k].ry, kShapes[k].mode>( \
+      p, fa, fb, flags, rho_m, ux_m, uy_m, wi, s)
+  LBM_SHAPE(0);
+  LBM_SHAPE(1);
+  LBM_SHAPE(2);
+  LBM_SHAPE(3);
+  LBM_SHAPE(4);
+  if constexpr (sizeof(typename Pop<S>::C) == 4) LBM_SHAPE(5);
+#undef LBM_SHAPE
+  return cudaErrorInvalidValue;
+}
+
+template <typename S>
+cudaError_t launch_tiles_s(int shape, const DevParams& p, const void* fa, void* fb,
+                           const uint8_t* flags, double* rho_m, double* ux_m, double* uy_m,
+                           const WallIn* wi, cudaStream_t s) {
+  switch (p.eos) {
+    case LBM_EOS_EXP:
+      return launch_tiles_t<S, LBM_EOS_EXP>(shape, p, fa, fb, flags, rho_m, ux_m, uy_m, wi, s);
+    case LBM_EOS_CS:
+      return launch_tiles_t<S, LBM_EOS_CS>(shape, p, fa, fb, flags, rho_m, ux_m, uy_m, wi, s);
+    default:
+      return launch_tiles_t<S, LBM_EOS_NONE>(shape, p, fa, fb, flags, rho_m, ux_m, uy_m, wi, s);
   }
 }
 
@@ -178,6 +250,51 @@ cudaError_t launch_batch_step(int precision, int eos, int ry, const BatchDomain*
   if (precision == LBM_FP16_DEV)
     return launch_batch_s<__half>(eos, ry, doms, tiles, n_tiles, claim, grid, s);
   return launch_batch_s<double>(eos, ry, doms, tiles, n_tiles, claim, grid, s);
+}
+
+// By nodes per SM (152), from us a step with the wall pass inside the step kernel / apart from it
+// (vector kernel, or scalar tiles where the width or format asks for them), droplet on a cylinder
+// (single phase in brackets):
+//   FP32  100^2 4.5 / 6.2 (4.2 / 5.0)   345^2 5.3 / 6.4 (4.6 / 5.6)   512^2 7.0 / 7.9 (5.8 / 6.3)
+//         724^2 9.2 / 12.2 (7.9 / 8.0)  1024^2 15.1 / 18.0 (11.3 / 11.2)  1448^2 33.7 / 36.1
+//         2048^2 61.6 / 58.0            2047^2 61.7 / 64.2 (scalar tiles apart)
+//   FP16  345^2 5.7 / 8.0               1024^2 16.7 / 16.9            2047^2 63.6 / 62.6
+//   FP64  100^2 9.7 / 21.7 (6.7 / 15.2) 300x350 30.1 / 39.8 (17.6 / 26.8)  1024^2 225.6 / 228.8
+// Few nodes want small tiles, so that every SM has some: FP64 100^2 9.7 (16 x 4), 9.9 (16 x 8), 13.5
+// (32 x 8), 22.7 us (32 x 16); 600^2 94.8, 84.6, 83.6, 86.0 us; FP32 400^2 6.1 (32 x 8, walls
+// inline), 6.7 (apart), 7.0 us (32 x 16), 600^2 10.0, 8.7, 8.1 us.
+int pick_step_tiles(int precision, int eos, int nx, int ny, int* tw, int* th) {
+  const long long per_sm = ((long long)nx * ny + 151) / 152;
+  const bool psi = eos != LBM_EOS_NONE, vec = step_vec_supported(precision, nx, ny);
+  int shape = -1;
+  if (precision == LBM_FP64) {
+    if (per_sm <= (psi ? 256 : 1024)) shape = 0;
+    else if (!psi || per_sm <= 2560) shape = 1;
+    else shape = 4;
+    // a second set of FP64 moments is 24 bytes a node: only where a step is short
+    if (per_sm > 16384) shape = -1;
+  } else if (per_sm <= (psi ? 1280 : (precision == LBM_FP16_DEV ? 2048 : 2560))) {
+    shape = 2;
+  } else if (psi || !vec) {
+    if (psi && per_sm <= 2048) shape = 3;
+    else if (per_sm <= 8192) shape = 4;
+    else if (precision == LBM_FP32_DEV) shape = !vec || per_sm <= 16384 ? 5 : -1;
+    else shape = !vec && per_sm <= 16384 ? 4 : -1;
+  }
+  if (shape < 0) return -1;
+  *tw = kShapes[shape].w;
+  *th = kShapes[shape].ty * kShapes[shape].ry;
+  return shape;
+}
+
+cudaError_t launch_step_tiles(int shape, int precision, const DevParams& p, const void* fa,
+                              void* fb, const uint8_t* flags, double* rho_m, double* ux_m,
+                              double* uy_m, const WallIn* wi, cudaStream_t s) {
+  if (precision == LBM_FP32_DEV)
+    return launch_tiles_s<float>(shape, p, fa, fb, flags, rho_m, ux_m, uy_m, wi, s);
+  if (precision == LBM_FP16_DEV)
+    return launch_tiles_s<__half>(shape, p, fa, fb, flags, rho_m, ux_m, uy_m, wi, s);
+  return launch_tiles_s<double>(shape, p, fa, fb, flags, rho_m, ux_m, uy_m, wi, s);
 }
 
 cudaError_t launch_step(int precision, const DevParams& p, const void* fa, void* fb,

@@ -1,6 +1,6 @@
 // Shared tile arithmetic of the step kernels (csrc/step.cu, csrc/step_tma.cu).
 #pragma once
-#include "d2q9.cuh"
+#include "wall_tile.cuh"
 
 namespace lbm {
 namespace step_core {
@@ -280,13 +280,19 @@ __device__ __forceinline__ void tile_phase2(const DevParams& p, void* __restrict
 // psi_s: shared memory of (TYN RY + 2) x (TXN + 2) values.
 // PDL: the caller is a kernel of a time step that has not waited for the one before yet; the
 // tile loads its flags first, then waits.
-template <typename S, int EOS, bool FIELDS, int RY, int TYN = TYT, int TXN = TX, bool PDL = false>
+// WALL: fa holds streamed values whose wall pass has not run; the tile (index t) applies it to what
+// it loads (wi; csrc/wall_tile.cuh; wall_smem: its shared memory): 1 while those loads are in
+// flight, 2 in a call before them.
+template <typename S, int EOS, bool FIELDS, int RY, int TYN = TYT, int TXN = TX, bool PDL = false,
+          int WALL = 0>
 __device__ __forceinline__ void step_tile(const DevParams& p, const void* __restrict__ fa,
                                           void* __restrict__ fb,
                                           const uint8_t* __restrict__ flags,
                                           double* __restrict__ rho_m, double* __restrict__ ux_m,
                                           double* __restrict__ uy_m, int x0, int y0,
-                                          typename Pop<S>::C (*psi_s)[TXN + 2]) {
+                                          typename Pop<S>::C (*psi_s)[TXN + 2],
+                                          const WallIn* wi = nullptr, int t = 0,
+                                          unsigned char* wall_smem = nullptr) {
   using C = typename StoreTraits<S>::C;
   constexpr bool DEV = StoreTraits<S>::deviation;
   constexpr int TH = TYN * RY;  // tile height in nodes
@@ -332,6 +338,32 @@ __device__ __forceinline__ void step_tile(const DevParams& p, const void* __rest
       }
     }
   };
+  const int c = ty * TXN + tx;  // thread index
+  wall::TileWalls<S, TXN * TYN> walls;
+  auto wall_begin = [&] {
+    if constexpr (WALL == 1) walls.begin(*wi, t, c, wall_smem);
+    if constexpr (WALL == 2) walls.head = wi->heads[t];
+  };
+  auto wall_apart = [&] {  // after the wait
+    if constexpr (WALL == 2) {
+      if (walls.head.w > 0) {
+        wall::tile_walls_apart<S, TXN * TYN>(p, *wi, fa, t, c, wall_smem);
+        walls.carve(*wi, wall_smem);
+      }
+    }
+  };
+  auto wall_run = [&] {  // and take the own nodes' values
+    if constexpr (WALL != 0) {
+      if constexpr (WALL == 1) walls.run(p, *wi, fa, c);
+#pragma unroll
+      for (int r = 0; r < RY; ++r)
+        // (without psi the tables hold the nodes that the tile owns only)
+        if ((fl[r] & (FLAG_SOLID | FLAG_BOUNDARY)) == FLAG_BOUNDARY &&
+            (EOS != LBM_EOS_NONE || (x < nx && y0 + ty + r * TYN < ny)))
+          walls.take(p, (ty + r * TYN + 1) * (TXN + 2) + tx + 1, f[r]);
+    }
+  };
+
   if constexpr (EOS != LBM_EOS_NONE) {
     // One-node ring around the tile, 2 (TX + 2) + 2 TH cells, one per thread of the first
     // kRing threads.  Its loads are issued first, then the own nodes' (the batched FP16 step ran
@@ -339,9 +371,8 @@ __device__ __forceinline__ void step_tile(const DevParams& p, const void* __rest
     // flight, so a CTA waits for memory once.
     constexpr int kRing = 2 * (TXN + 2) + 2 * TH;
     static_assert(kRing <= TXN * TYN, "one ring cell per thread");
-    const int c = ty * TXN + tx;
     int hx = 0, hy = 0, ring_node = 0;
-    bool ring_fluid = false;
+    bool ring_fluid = false, ring_bnd = false;
     C v[9];
     if (c < kRing) {
       if (c < 2 * (TXN + 2)) {
@@ -362,12 +393,16 @@ __device__ __forceinline__ void step_tile(const DevParams& p, const void* __rest
         gy = gy < 0 ? gy + ny : (gy >= ny ? gy - ny : gy);
       }
       const int m = gy * nx + gx;
-      ring_fluid = ring_need && !(flags[LBM_CHK(m, N)] & FLAG_SOLID);
+      const uint8_t rf = flags[LBM_CHK(m, N)];
+      ring_fluid = ring_need && !(rf & FLAG_SOLID);
+      ring_bnd = ring_fluid && (rf & FLAG_BOUNDARY);
       ring_node = m;
     }
     if constexpr (PDL) {
       load_own_flags();
+      wall_begin();
       pdl_wait();
+      wall_apart();
     }
     if (ring_fluid) {
 #pragma unroll
@@ -375,6 +410,10 @@ __device__ __forceinline__ void step_tile(const DevParams& p, const void* __rest
     }
     if constexpr (!PDL) load_own_flags();
     load_own();
+    wall_run();
+    if constexpr (WALL != 0) {
+      if (ring_bnd) walls.take(p, hy * (TXN + 2) + hx, v);
+    }
 #pragma unroll
     for (int r = 0; r < RY; ++r) {
       if (!(fl[r] & FLAG_SOLID)) rho[r] = density_of<DEV>(rho_ref, f[r]);
@@ -386,8 +425,11 @@ __device__ __forceinline__ void step_tile(const DevParams& p, const void* __rest
     __syncthreads();
   } else {
     load_own_flags();
+    wall_begin();
     if constexpr (PDL) pdl_wait();
+    wall_apart();
     load_own();
+    wall_run();
 #pragma unroll
     for (int r = 0; r < RY; ++r)
       if (!(fl[r] & FLAG_SOLID)) rho[r] = density_of<DEV>(rho_ref, f[r]);

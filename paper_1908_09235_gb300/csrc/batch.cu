@@ -43,6 +43,7 @@ struct lbm_batch {
   std::vector<lbm_tune_trial> trials;  // of the last lbm_batch_tune
   int step_grid = 0, bnd_grid = 0;
   bool dirty = true;
+  bool behind = false;  // steps were launched since h_doms was last brought up to date
   cudaGraphExec_t graph = nullptr;
   int graph_steps = 16;
   lbm_status status = LBM_OK;
@@ -99,9 +100,11 @@ void drop_graph(lbm_batch* b) {
   }
 }
 
-// Bring cur / steps_left / steps_done of every lattice from the device into h_doms.
+// Bring cur / steps_left / steps_done of every lattice from the device into h_doms.  Only steps
+// change them, so calls between two steps share one copy: reading out 512 lattices took 512 copies
+// of the whole table, 17-30 ms beside 174 ms for 200 steps.
 lbm_status sync_down(lbm_batch* b) {
-  if (!b->d_doms) return LBM_OK;
+  if (!b->d_doms || !b->behind) return LBM_OK;
   std::vector<BatchDomain> tmp(b->max_domains);
   BCUDA(b, cudaMemcpyAsync(tmp.data(), b->d_doms, sizeof(BatchDomain) * b->max_domains,
                            cudaMemcpyDeviceToHost, b->stream));
@@ -114,6 +117,7 @@ lbm_status sync_down(lbm_batch* b) {
     b->slots[d]->cur = tmp[d].cur;
     b->slots[d]->steps = tmp[d].steps_done;
   }
+  b->behind = false;
   return LBM_OK;
 }
 
@@ -146,6 +150,8 @@ int* claim_counter(lbm_batch* b) {
 // of a lattice stand together in row-major order; the lattices follow in slot order, or by tile
 // count, largest first, for LBM_SCHED_CLAIM_LARGEST_FIRST (ties in slot order).
 lbm_status upload_tables(lbm_batch* b) {
+  const lbm_status down = sync_down(b);  // the whole table goes up: with the current state
+  if (down != LBM_OK) return down;
   const int TH = batch_tile_rows(b->ry), TW = batch_tile_cols();
   std::vector<int> order;
   for (int d = 0; d < b->max_domains; ++d)
@@ -346,6 +352,7 @@ lbm_status lbm_batch_step(lbm_batch* b, int32_t n) {
   if (!b || n < 0) return LBM_EINVAL;
   lbm_status st = ready(b);
   if (st != LBM_OK) return st;
+  b->behind = b->behind || n > 0;
   while (n >= b->graph_steps) {
     if (!b->graph) {
       cudaGraph_t g = nullptr;
@@ -373,6 +380,7 @@ lbm_status lbm_batch_step_timed(lbm_batch* b, int32_t n, double* ms_total, doubl
   if (!b || n < 1) return LBM_EINVAL;
   lbm_status st = ready(b);
   if (st != LBM_OK) return st;
+  b->behind = true;
   std::vector<cudaEvent_t> ev(2 * (size_t)n + 1);
   for (auto& e : ev) BCUDA(b, cudaEventCreate(&e));
   BCUDA(b, cudaEventRecord(ev[0], b->stream));

@@ -185,32 +185,20 @@ struct InPlace {
   __device__ __forceinline__ void carry(int b, double c) const { out[b] = c; }
 };
 
-// Channel ends (Sec. 4.2), after streaming and the wall pass; one thread per row j.  Inlet
-// i = 0: the populations entering from the left (1, 5, 8) follow from the prescribed velocity
-// (u_in, 0) and the known ones by Zou and He's rule:
-//   rho = (f0 + f2 + f4 + 2 (f3 + f6 + f7)) / (1 - u_in),  f1 = f3 + 2/3 rho u_in,
-//   f5 = f7 - (f2 - f4)/2 + rho u_in / 6,  f8 = f6 + (f2 - f4)/2 + rho u_in / 6.
-// Outlet i = nx - 1 (fully developed flow): the populations entering from the right (3, 6, 7)
-// equal those of column nx - 2.  FP64 arithmetic on the full populations (deviation + w rho_ref).
+// Channel ends (Sec. 4.2), after streaming and the wall pass; one thread per row j: the inlet at
+// i = 0, and at the outlet i = nx - 1 (fully developed flow) the populations entering from the right
+// (3, 6, 7) equal those of column nx - 2.
 template <typename S>
 __device__ __forceinline__ void open_row(const DevParams& p, int j, void* __restrict__ fb,
                                          const uint8_t* __restrict__ flags, double u_in) {
   const int nx = p.nx, N = p.N;
-  const double rr = p.rho_ref;
   const bool in = j < p.ny;
   const int n0 = in ? j * nx : 0, n1 = n0 + nx - 1;
   const bool fluid0 = in && !(flags[n0] & FLAG_SOLID), fluid1 = in && !(flags[n1] & FLAG_SOLID);
   pdl_wait();
-  auto get = [&](int a, int n) { return Pop<S>::load_e(fb, a * N + n, N) + wgt<double>(a) * rr; };
-  auto put = [&](int a, int n, double v) { Pop<S>::store_e(fb, a * N + n, N, v - wgt<double>(a) * rr); };
-  if (fluid0) {
-    const double f0 = get(0, n0), f2 = get(2, n0), f3 = get(3, n0), f4 = get(4, n0);
-    const double f6 = get(6, n0), f7 = get(7, n0);
-    const double rho = (f0 + f2 + f4 + 2.0 * (f3 + f6 + f7)) / (1.0 - u_in);
-    put(1, n0, f3 + 2.0 / 3.0 * rho * u_in);
-    put(5, n0, f7 - 0.5 * (f2 - f4) + rho * u_in / 6.0);
-    put(8, n0, f6 + 0.5 * (f2 - f4) + rho * u_in / 6.0);
-  }
+  if (fluid0)
+    inlet(p.rho_ref, u_in, [&](int a) { return Pop<S>::load_e(fb, a * N + n0, N); },
+          [&](int a, double v) { Pop<S>::store_e(fb, a * N + n0, N, v); });
   if (fluid1) {
     // copies of stored values: no rounding for any format
     Pop<S>::store_e(fb, 3 * N + n1, N, Pop<S>::load_e(fb, 3 * N + n1 - 1, N));

@@ -111,10 +111,11 @@ lbm_status launch_one_step(lbm_ctx* c, cudaStream_t s, int cur) {
   return launch_walls(c, s, cur);
 }
 
-// The wall pass of a step can be done by the next step's kernel (Zhao-Yong's reads the lattice that
-// kernel overwrites; the channel ends come after the wall pass).
+// The wall pass of a step, and the channel ends where they touch other nodes, can be done by the next
+// step's kernel (but Zhao-Yong's wall pass reads the lattice which that kernel overwrites).
 bool walls_in_steps(const lbm_ctx* c) {
-  return c->tiles_shape >= 0 && c->nb > 0 && !c->open_x && c->p.scheme != LBM_ZHAO_YONG;
+  return c->tiles_shape >= 0 && c->nb > 0 && (!c->open_x || c->ends_with_wall) &&
+         c->p.scheme != LBM_ZHAO_YONG;
 }
 
 // n steps from lattice cur, launched one after the other.  Where walls_in_steps, every kernel but
@@ -137,6 +138,8 @@ lbm_status launch_steps(lbm_ctx* c, cudaStream_t s, int cur, int n) {
     wi.uy = macro[1 - m][2];
     wi.carry_in = carry[1 - m];
     wi.carry_out = carry[m];
+    wi.open_x = c->open_x ? 1 : 0;
+    wi.u_in = c->u_in;
     const cudaError_t e =
         launch_step_tiles(c->tiles_shape, c->precision, c->p, c->f[cur], c->f[1 - cur], c->flags,
                           macro[m][0], macro[m][1], macro[m][2], k > 0 ? &wi : nullptr, s);

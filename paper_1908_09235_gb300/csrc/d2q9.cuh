@@ -104,7 +104,13 @@ struct Pop<double> {
   static __device__ __forceinline__ C load(const void* b, int a, int N, int n) {
     return __ldcg(static_cast<const double*>(b) + a * N + LBM_CHK(n, N));
   }
+  // through L1, for kernels launched in plain stream order
+  static __device__ __forceinline__ C load_l1(const void* b, int a, int N, int n) {
+    return static_cast<const double*>(b)[a * N + LBM_CHK(n, N)];
+  }
   static __device__ __forceinline__ C rounded(int a, C v) { return v; }
+  // an FP64 value as stored in plane a
+  static __device__ __forceinline__ C rounded_e(int a, double v) { return v; }
   static __device__ __forceinline__ void store(void* b, int a, int N, int n, C v) {
     static_cast<double*>(b)[a * N + LBM_CHK(n, N)] = v;
   }
@@ -131,7 +137,11 @@ struct Pop<float> {
   static __device__ __forceinline__ C load(const void* b, int a, int N, int n) {
     return __ldcg(static_cast<const float*>(b) + a * N + LBM_CHK(n, N));
   }
+  static __device__ __forceinline__ C load_l1(const void* b, int a, int N, int n) {
+    return static_cast<const float*>(b)[a * N + LBM_CHK(n, N)];
+  }
   static __device__ __forceinline__ C rounded(int a, C v) { return v; }
+  static __device__ __forceinline__ C rounded_e(int a, double v) { return float(v); }
   static __device__ __forceinline__ void store(void* b, int a, int N, int n, C v) {
     static_cast<float*>(b)[a * N + LBM_CHK(n, N)] = v;
   }
@@ -166,8 +176,15 @@ struct Pop<__half> {
     return a == 0 ? __ldcg(static_cast<const float*>(b) + n)
                   : __half2float(__ldcg(moving(b, N) + (a - 1) * N + n));
   }
+  static __device__ __forceinline__ C load_l1(const void* b, int a, int N, int n) {
+    n = LBM_CHK(n, N);
+    return a == 0 ? static_cast<const float*>(b)[n] : __half2float(moving(b, N)[(a - 1) * N + n]);
+  }
   static __device__ __forceinline__ C rounded(int a, C v) {
     return a == 0 ? v : __half2float(__float2half_rn(v));
+  }
+  static __device__ __forceinline__ C rounded_e(int a, double v) {
+    return a == 0 ? float(v) : __half2float(__double2half(v));
   }
   static __device__ __forceinline__ void store(void* b, int a, int N, int n, C v) {
     n = LBM_CHK(n, N);

@@ -160,6 +160,8 @@ struct WallIn {
   const double *rho, *ux, *uy;  // the moments that the step before stored
   const double* carry_in;       // the FP64 residues before and after
   double* carry_out;
+  int open_x;  // the channel ends too (single phase; they and the walls touch different nodes)
+  double u_in;
 };
 
 // One lattice of a batch as the batched kernels see it.  cur and steps_left are advanced on

@@ -260,6 +260,8 @@ cudaError_t launch_batch_step(int precision, int eos, int ry, const BatchDomain*
 //         2048^2 61.6 / 58.0            2047^2 61.7 / 64.2 (scalar tiles apart)
 //   FP16  345^2 5.7 / 8.0               1024^2 16.7 / 16.9            2047^2 63.6 / 62.6
 //   FP64  100^2 9.7 / 21.7 (6.7 / 15.2) 300x350 30.1 / 39.8 (17.6 / 26.8)  1024^2 225.6 / 228.8
+// (The same in the vector kernel's tiles lost where it is the faster one: its registers leave no room,
+// 4096^2 FP32 207.9 / 199.9, FP16 192.4 / 187.8, single-phase FP16 139.1 / 124.1.)
 // Few nodes want small tiles, so that every SM has some: FP64 100^2 9.7 (16 x 4), 9.9 (16 x 8), 13.5
 // (32 x 8), 22.7 us (32 x 16); 600^2 94.8, 84.6, 83.6, 86.0 us; FP32 400^2 6.1 (32 x 8, walls
 // inline), 6.7 (apart), 7.0 us (32 x 16), 600^2 10.0, 8.7, 8.1 us.

@@ -324,6 +324,9 @@ __device__ __forceinline__ void step_tile(const DevParams& p, const void* __rest
       fl[r] = (x <= nx && y0 + ty + r * TYN <= ny) ? flags[LBM_CHK(own_node(r), N)]
                                                    : uint8_t(FLAG_SOLID);
   };
+  auto load = [&](int a, int n) {
+    if constexpr (PDL) return Pop<S>::load(fa, a, N, n); else return Pop<S>::load_l1(fa, a, N, n);
+  };
   auto load_own = [&] {
 #pragma unroll
     for (int r = 0; r < RY; ++r) {
@@ -331,7 +334,7 @@ __device__ __forceinline__ void step_tile(const DevParams& p, const void* __rest
       rho[r] = C(1);
       if (!(fl[r] & FLAG_SOLID)) {
 #pragma unroll
-        for (int a = 0; a < 9; ++a) f[r][a] = Pop<S>::load(fa, a, N, n);
+        for (int a = 0; a < 9; ++a) f[r][a] = load(a, n);
       } else {
 #pragma unroll
         for (int a = 0; a < 9; ++a) f[r][a] = C(0);
@@ -361,6 +364,19 @@ __device__ __forceinline__ void step_tile(const DevParams& p, const void* __rest
         if ((fl[r] & (FLAG_SOLID | FLAG_BOUNDARY)) == FLAG_BOUNDARY &&
             (EOS != LBM_EOS_NONE || (x < nx && y0 + ty + r * TYN < ny)))
           walls.take(p, (ty + r * TYN + 1) * (TXN + 2) + tx + 1, f[r]);
+      if constexpr (EOS == LBM_EOS_NONE) {
+        if (wi->open_x && (x == 0 || x == nx - 1)) {
+#pragma unroll
+          for (int r = 0; r < RY; ++r) {
+            if (fl[r] & FLAG_SOLID) continue;
+            if (x == 0)
+              wall::inlet(p.rho_ref, wi->u_in, [&](int a) { return double(f[r][a]); },
+                          [&](int a, double v) { f[r][a] = Pop<S>::rounded_e(a, v); });
+            else
+              for (int a : {3, 6, 7}) f[r][a] = Pop<S>::load(fa, a, N, own_node(r) - 1);
+          }
+        }
+      }
     }
   };
 
@@ -406,7 +422,7 @@ __device__ __forceinline__ void step_tile(const DevParams& p, const void* __rest
     }
     if (ring_fluid) {
 #pragma unroll
-      for (int a = 0; a < 9; ++a) v[a] = Pop<S>::load(fa, a, N, ring_node);
+      for (int a = 0; a < 9; ++a) v[a] = load(a, ring_node);
     }
     if constexpr (!PDL) load_own_flags();
     load_own();

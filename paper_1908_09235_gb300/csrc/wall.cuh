@@ -194,6 +194,23 @@ __device__ __forceinline__ T rest_value(T f0_d, double dm, double residue, doubl
   return st;
 }
 
+// Inlet of the channel mode (Sec. 4.2) at a node of column 0: the populations entering from the left
+// (1, 5, 8) follow from the prescribed velocity (u_in, 0) and the known ones by Zou and He's rule,
+//   rho = (f0 + f2 + f4 + 2 (f3 + f6 + f7)) / (1 - u_in),  f1 = f3 + 2/3 rho u_in,
+//   f5 = f7 - (f2 - f4)/2 + rho u_in / 6,  f8 = f6 + (f2 - f4)/2 + rho u_in / 6,
+// in FP64 on the full populations (stored value + w rho_ref); get(a): the stored value, put(a, v):
+// the new one, to be rounded to the format.
+template <typename Get, typename Set>
+__device__ __forceinline__ void inlet(double rho_ref, double u_in, Get get, Set set) {
+  auto whole = [&](int a) { return get(a) + wgt<double>(a) * rho_ref; };
+  const double f0 = whole(0), f2 = whole(2), f3 = whole(3), f4 = whole(4), f6 = whole(6),
+               f7 = whole(7);
+  const double rho = (f0 + f2 + f4 + 2.0 * (f3 + f6 + f7)) / (1.0 - u_in);
+  set(1, f3 + 2.0 / 3.0 * rho * u_in - wgt<double>(1) * rho_ref);
+  set(5, f7 - 0.5 * (f2 - f4) + rho * u_in / 6.0 - wgt<double>(5) * rho_ref);
+  set(8, f6 + 0.5 * (f2 - f4) + rho * u_in / 6.0 - wgt<double>(8) * rho_ref);
+}
+
 // The wall values of a boundary node by the 8 lanes of its group, lane k one link (node_ok false: a
 // padding group, which still takes part in the shuffles).  put.incoming(dst, a, v) and
 // put.rest(n, v) take the unknown population f_a(x_b, t+1) and the corrected rest population and

@@ -89,3 +89,19 @@ def test_every_tile_shape_gives_the_bits_of_the_wall_kernel(gpu_lib, precision, 
         # a graph of 32 steps and a remainder
         assert _same(_run([35], *args, 0, kind, circles, False),
                      _run([35], *args, 1, kind, circles, False)), scheme
+
+
+@pytest.mark.parametrize("precision", [lbm.FP64, lbm.FP32_DEV, lbm.FP16_DEV])
+@pytest.mark.parametrize("nx,ny", [(120, 64), (121, 75), (800, 500)])
+def test_channel_ends_in_the_tiles_give_the_bits_of_their_kernel(gpu_lib, precision, nx, ny):
+    def run(path):
+        lat = lbm.Lattice(nx, ny, 0.8, "mod_b", circles=[(0.4 * nx, 0.5 * ny, 0.1 * ny)],
+                          eos=lbm.make_eos(lbm.EOS_NONE), precision=precision, kernel_path=path)
+        lat.init_fields(np.ones(nx * ny), np.full(nx * ny, 0.05))
+        lat.set_inflow(0.05)
+        lat.step(35)
+        out = [np.nan_to_num(a, nan=-7.0) for a in lat.fields()] + [np.array(lat.force())]
+        lat.close()
+        return out
+
+    assert _same(run(0), run(1))

@@ -128,7 +128,9 @@ typedef struct {
                         * 0: the fastest measured.  Small and mid-size lattices: scalar tiles   *
                         *    sized to the lattice that also do the wall pass of the step before  *
                         *    (the last step's stays a launch of its own; not for Zhao-Yong links *
-                        *    and open channels).  Others, with FP32/FP16 deviations, nx % 4 == 0 *
+                        *    and some open channels).  Large two-phase FP16 lattices with        *
+                        *    nx % 8 == 0: a kernel whose warps march up strips of rows brought  *
+                        *    by tensor copies.  Others, with FP32/FP16 deviations, nx % 4 == 0 *
                         *    and ny >= 8 (FP16: 12) the vectorised kernel (population vectors   *
                         *    of 16 B; the two psi-ring rows of tiles away from the x seam staged *
                         *    by tensor copies (TMA), the rest of the halo by cp.async), otherwise *

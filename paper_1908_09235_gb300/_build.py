@@ -17,7 +17,7 @@ LIBDIR = os.path.join(HERE, "_lib")
 LIB = os.path.join(LIBDIR, "liblbm_gb300.so")
 CHECKED_LIB = os.path.join(LIBDIR, "liblbm_gb300_checked.so")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
-CUDA_SOURCES = ["step.cu", "step_vec.cu", "step_tma.cu", "boundary.cu", "geometry.cu",
+CUDA_SOURCES = ["step.cu", "step_vec.cu", "step_march.cu", "step_tma.cu", "boundary.cu", "geometry.cu",
                 "ledger.cu", "capi.cu", "batch.cu", "mass_noalloc.cu", "probe.cu"]
 CXX_SOURCES = ["eos_host.cpp"]
 

@@ -96,13 +96,19 @@ cudaError_t launch_step_vec(int precision, const DevParams& p, const void* fa, v
                             const uint8_t* flags, double* rho_m, double* ux_m, double* uy_m,
                             bool fields_only, cudaStream_t s, bool tma_ring = false,
                             int* err = nullptr);
-// path: 0 = the vectorised kernel for the deviation formats where step_vec_supported(), else
-// the scalar tile kernel; 1 = the scalar tile kernel; 3 = the vectorised kernel where
+// path: 0 = for the deviation formats the marching kernel where step_march_supported(), the
+// vectorised kernel where step_vec_supported(), else the scalar tile kernel; 1 = the scalar tile kernel; 3 = the vectorised kernel where
 // step_vec_supported() (FP64 too), its psi ring staged by cp.async only; 4 = as 0.  Paths 0 and
 // 4 stage the deviation kernels' psi-ring rows by tensor copies where a tile allows (needs err)
 cudaError_t launch_step(int precision, const DevParams& p, const void* fa, void* fb,
                         const uint8_t* flags, double* rho_m, double* ux_m, double* uy_m,
                         bool fields_only, cudaStream_t s, int path = 0, int* err = nullptr);
+
+// The marching kernel of large two-phase FP16 lattices (csrc/step_march.cu); an expired wait sets
+// kErrTimeout in *err.
+bool step_march_supported(int precision, int eos, int nx, int ny);
+cudaError_t launch_step_march(const DevParams& p, const void* fa, void* fb, const uint8_t* flags,
+                              double* rho_m, double* ux_m, double* uy_m, int* err, cudaStream_t s);
 
 // The scalar tiles in the shapes of small lattices, whose step kernels can apply the previous
 // step's wall pass themselves (wi; nullptr: a plain step).  pick_step_tiles: the shape for a

@@ -302,6 +302,9 @@ cudaError_t launch_step_tiles(int shape, int precision, const DevParams& p, cons
 cudaError_t launch_step(int precision, const DevParams& p, const void* fa, void* fb,
                         const uint8_t* flags, double* rho_m, double* ux_m, double* uy_m,
                         bool fields_only, cudaStream_t s, int path, int* err) {
+  if ((path == 0 || path == 4) && !fields_only && err &&
+      step_march_supported(precision, p.eos, p.nx, p.ny))
+    return launch_step_march(p, fa, fb, flags, rho_m, ux_m, uy_m, err, s);
   // FP64 is bound by the FP64 pipe, where the scalar tiling (fewer ring psi per node) is faster
   const bool vec = path == 3 || ((path == 0 || path == 4) && precision != LBM_FP64);
   if (vec && step_vec_supported(precision, p.nx, p.ny))

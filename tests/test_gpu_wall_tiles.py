@@ -105,3 +105,17 @@ def test_channel_ends_in_the_tiles_give_the_bits_of_their_kernel(gpu_lib, precis
         return out
 
     assert _same(run(0), run(1))
+
+
+@pytest.mark.parametrize("nx,ny,kind", [(128, 9740, "cs"), (136, 9161, "exp"), (8, 65530, "cs"),
+                                        (1048, 1189, "cs"), (1272, 1000, "exp")])
+def test_the_marching_kernel_gives_the_bits_of_the_scalar_tiles(gpu_lib, nx, ny, kind):
+    # FP16 lattices just above the size from which kernel_path 0 and 4 march: whole strips, a last
+    # strip of one lane or 30, one strip of two lanes (its left and right neighbours itself), and
+    # heights that are no multiple of a strip's rows; seven steps and their wall pass
+    circles = [(0.5 * nx, 0.35 * ny, 0.2 * nx)] if nx > 8 else []
+    for scheme in ("mod_b", "zhao_yong"):
+        args = (nx, ny, lbm.FP16_DEV, scheme)
+        a = _run([7], *args, 4, kind, circles, False)
+        b = _run([7], *args, 1, kind, circles, False)
+        assert _same(a[:3], b[:3]) and a[-1] == b[-1], scheme

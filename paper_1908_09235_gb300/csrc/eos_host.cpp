@@ -135,6 +135,13 @@ static void fill(Consts<C>& k, const DevParams& p) {
   k.h3 = C(1.5 * (1.0 - p.omega));
   k.h12 = C(6.0 * (1.0 - p.omega));
   k.gF = C(2.0 - 0.5 * p.omega);
+  const double w[2] = {1.0 / 9.0, 1.0 / 36.0};
+  for (int c = 0; c < 2; ++c) {
+    k.wo45[c] = C(w[c] * 4.5 * p.omega);
+    k.wo3[c] = C(w[c] * 3.0 * p.omega);
+    k.wK3[c] = C(w[c] * 9.0 * p.guo_pref);
+    k.wK[c] = C(w[c] * 3.0 * p.guo_pref);
+  }
   k.gw1 = C(-p.G / 3.0);
   k.gw5 = C(-p.G / 12.0);
   k.G = C(p.G);

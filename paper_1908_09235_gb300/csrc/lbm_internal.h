@@ -23,9 +23,12 @@ enum : uint8_t {
 template <typename C>
 struct Consts {
   C omega, one_m_omega, K;     // 1/tau, 1 - 1/tau, 3 (1 - 1/(2 tau))
-  // FP64 collision: h = (1 - omega)/2 (h1), h/(3 w) for the axis (h3 = 3 h) and the diagonals
+  // FP64 two-phase collision: h = (1 - omega)/2 (h1), h/(3 w) for the axis (h3 = 3 h) and the diagonals
   // (h12 = 12 h), gF = 2 - omega/2; and the force weights with -G folded in: -G/3, -G/12
   C h1, h3, h12, gF;
+  // FP64 single-phase collision, per weight class c (0: axis, w = 1/9; 1: diagonal, w = 1/36):
+  // w 4.5 omega, w 3 omega, w 3 K, w K
+  C wo45[2], wo3[2], wK3[2], wK[2];
   C gw1, gw5;
   C G, psi0, rho0, a, b4, RT, two_over_G, psi_wall;
   C gx, gy, azC, azcx, azcy;

@@ -19,10 +19,10 @@ struct StoreTraits {
 // Sum of the nine stored values in direction order (a node's density, less rho_ref for the
 // deviation format).  Own nodes and ring nodes use the same arithmetic, so every CTA that needs
 // psi of a node computes the same value.
-// FP64 adds opposite directions first: the collision uses those four sums again.
-template <typename C>
+// FP64 with a pseudopotential adds opposite directions first: its collision uses those four sums.
+template <int EOS, typename C>
 __device__ __forceinline__ C pop_sum(const C (&f)[9]) {
-  if constexpr (sizeof(typename Elem<C>::C) == 8) {
+  if constexpr (sizeof(typename Elem<C>::C) == 8 && EOS != LBM_EOS_NONE) {
     return r_add(f[0], r_add(r_add(r_add(f[1], f[3]), r_add(f[2], f[4])),
                              r_add(r_add(f[5], f[7]), r_add(f[6], f[8]))));
   } else {
@@ -35,12 +35,12 @@ __device__ __forceinline__ C pop_sum(const C (&f)[9]) {
 
 // A node's density from its nine stored values: their sum, plus rho_ref for the deviation
 // formats (FP64 storage holds the populations themselves).
-template <bool DEV, typename L>
+template <bool DEV, int EOS, typename L>
 __device__ __forceinline__ L density_of(typename Elem<L>::C rho_ref, const L (&f)[9]) {
   if constexpr (DEV)
-    return r_add(splat<L>(rho_ref), pop_sum<L>(f));
+    return r_add(splat<L>(rho_ref), pop_sum<EOS>(f));
   else
-    return pop_sum<L>(f);
+    return pop_sum<EOS>(f);
 }
 
 // A post-collision value rounded to the storage format of plane a (per element).  Node pairs of
@@ -106,7 +106,7 @@ __device__ __forceinline__ void collide_node(const DevParams& p,
     }
   }
   L out[9];
-  if constexpr (sizeof(C) == 8) {
+  if constexpr (sizeof(C) == 8 && EOS != LBM_EOS_NONE) {
     // FP64 arithmetic is bound by the FP64 pipe (2 operations per clock and SM), so this form has
     // the fewest operations.  With j = m + F/2 = rho u (m: the momentum of g), k = 1 - 1/(2 tau),
     //   G = omega j + 2 k F = omega m + (2 - omega/2) F,   H = omega j + k F = omega m + F,
@@ -119,7 +119,6 @@ __device__ __forceinline__ void collide_node(const DevParams& p,
     const L d1 = r_sub(g[1], g[3]), d2 = r_sub(g[2], g[4]);
     const L d5 = r_sub(g[5], g[7]), d8 = r_sub(g[8], g[6]);
     const L mx = r_add(r_add(d1, d5), d8), my = r_sub(r_add(d2, d5), d8);
-    if constexpr (EOS == LBM_EOS_NONE) inv = q_rcp(rh);
     ux = r_mul(r_fma(0.5, Fx, mx), inv);
     uy = r_mul(r_fma(0.5, Fy, my), inv);
     const L omx = r_mul(k.omega, mx), omy = r_mul(k.omega, my);
@@ -168,20 +167,45 @@ __device__ __forceinline__ void collide_node(const DevParams& p,
     // the even part P = A0 + (4.5 rho omega eu + 3 K eF) eu and the odd part Q = 3 rho omega eu +
     // K eF.
     out[0] = r_fma(one_m_omega, g[0], r_mul(c_(wgt<C>(0)), A0));
-    // FP32 arithmetic (issue- and register-bound kernels): fewer live values per node
-    const L orho = r_mul(c_(k.omega), rh);
-    const L o45 = r_mul(c_(C(4.5)), orho), o3 = r_mul(c_(C(3)), orho);
-    const L K = c_(k.K), K3 = r_mul(c_(C(3)), K);
+    if constexpr (sizeof(C) == 8) {
+      // FP64 single phase: w folded into coefficients per weight class c (axis, diagonal), al = w 4.5
+      // omega rho, be = w 3 omega rho, Aw = w A0 and the constants w 3 K, w K.  (The two-phase form
+      // above has fewer operations, but a single-phase flow's velocities decay to where another rounding
+      // is all of the difference, and they keep their bits.)
+      L al[2], be[2], Aw[2];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int a = i == 0 ? 1 : (i == 1 ? 2 : (i == 2 ? 5 : 6)), ab = opposite(a);
-      const L eu = i == 0 ? ux : (i == 1 ? uy : (i == 2 ? r_add(ux, uy) : r_sub(uy, ux)));
-      const L eF = i == 0 ? Fx : (i == 1 ? Fy : (i == 2 ? r_add(Fx, Fy) : r_sub(Fy, Fx)));
-      const L P = r_fma(r_fma(o45, eu, r_mul(K3, eF)), eu, A0);
-      const L Q = r_fma(o3, eu, r_mul(K, eF));
-      const L w = c_(wgt<C>(a));
-      out[a] = r_fma(one_m_omega, g[a], r_mul(w, r_add(P, Q)));
-      out[ab] = r_fma(one_m_omega, g[ab], r_mul(w, r_sub(P, Q)));
+      for (int c = 0; c < 2; ++c) {
+        al[c] = r_mul(c_(k.wo45[c]), rh);
+        be[c] = r_mul(c_(k.wo3[c]), rh);
+        Aw[c] = r_mul(c_(wgt<C>(c == 0 ? 1 : 5)), A0);
+      }
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int a = i == 0 ? 1 : (i == 1 ? 2 : (i == 2 ? 5 : 6)), ab = opposite(a), c = i >> 1;
+        // e_a = (1,0), (0,1), (1,1), (-1,1)
+        const L eu = i == 0 ? ux : (i == 1 ? uy : (i == 2 ? r_add(ux, uy) : r_sub(uy, ux)));
+        const L eF = i == 0 ? Fx : (i == 1 ? Fy : (i == 2 ? r_add(Fx, Fy) : r_sub(Fy, Fx)));
+        const L wP = r_fma(r_fma(al[c], eu, r_mul(c_(k.wK3[c]), eF)), eu, Aw[c]);
+        const L wQ = r_fma(be[c], eu, r_mul(c_(k.wK[c]), eF));
+        out[a] = r_fma(one_m_omega, g[a], r_add(wP, wQ));
+        out[ab] = r_fma(one_m_omega, g[ab], r_sub(wP, wQ));
+      }
+    } else {
+      // FP32 arithmetic (issue- and register-bound kernels): fewer live values per node
+      const L orho = r_mul(c_(k.omega), rh);
+      const L o45 = r_mul(c_(C(4.5)), orho), o3 = r_mul(c_(C(3)), orho);
+      const L K = c_(k.K), K3 = r_mul(c_(C(3)), K);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int a = i == 0 ? 1 : (i == 1 ? 2 : (i == 2 ? 5 : 6)), ab = opposite(a);
+        const L eu = i == 0 ? ux : (i == 1 ? uy : (i == 2 ? r_add(ux, uy) : r_sub(uy, ux)));
+        const L eF = i == 0 ? Fx : (i == 1 ? Fy : (i == 2 ? r_add(Fx, Fy) : r_sub(Fy, Fx)));
+        const L P = r_fma(r_fma(o45, eu, r_mul(K3, eF)), eu, A0);
+        const L Q = r_fma(o3, eu, r_mul(K, eF));
+        const L w = c_(wgt<C>(a));
+        out[a] = r_fma(one_m_omega, g[a], r_mul(w, r_add(P, Q)));
+        out[ab] = r_fma(one_m_omega, g[ab], r_mul(w, r_sub(P, Q)));
+      }
     }
   }
 #pragma unroll
@@ -432,12 +456,12 @@ __device__ __forceinline__ void step_tile(const DevParams& p, const void* __rest
     }
 #pragma unroll
     for (int r = 0; r < RY; ++r) {
-      if (!(fl[r] & FLAG_SOLID)) rho[r] = density_of<DEV>(rho_ref, f[r]);
+      if (!(fl[r] & FLAG_SOLID)) rho[r] = density_of<DEV, EOS>(rho_ref, f[r]);
       const C ps = psi_own<C, EOS>(k, rho[r], inv[r]);
       psi_s[ty + r * TYN + 1][tx + 1] = (fl[r] & FLAG_SOLID) ? psi_w : ps;
     }
     if (c < kRing)
-      psi_s[hy][hx] = ring_fluid ? psi_of<C, EOS>(k, density_of<DEV>(rho_ref, v)) : psi_w;
+      psi_s[hy][hx] = ring_fluid ? psi_of<C, EOS>(k, density_of<DEV, EOS>(rho_ref, v)) : psi_w;
     __syncthreads();
   } else {
     load_own_flags();
@@ -448,7 +472,7 @@ __device__ __forceinline__ void step_tile(const DevParams& p, const void* __rest
     wall_run();
 #pragma unroll
     for (int r = 0; r < RY; ++r)
-      if (!(fl[r] & FLAG_SOLID)) rho[r] = density_of<DEV>(rho_ref, f[r]);
+      if (!(fl[r] & FLAG_SOLID)) rho[r] = density_of<DEV, EOS>(rho_ref, f[r]);
   }
 
   if constexpr (PDL) pdl_trigger();

@@ -127,7 +127,7 @@ __global__ void __launch_bounds__(32, kWarps)
 #pragma unroll
     for (int a = 0; a < 9; ++a) g[a] = Pop<S>::load(fa, a, N, n);
     side = (flags[LBM_CHK(n, N)] & FLAG_SOLID) ? psi_w
-                                               : psi_of<float, EOS>(k, density_of<true>(rho_ref, g));
+                                               : psi_of<float, EOS>(k, density_of<true, EOS>(rho_ref, g));
   }
 
   // psi of a row: [0] left neighbour, [1 .. 4] own, [5] right neighbour; and the own densities

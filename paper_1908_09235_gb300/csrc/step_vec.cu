@@ -474,7 +474,7 @@ __global__ void __launch_bounds__(VW* Vec<S>::VH, Vec<S>::kBlocks)
   L rho[NP], inv[NP];
 #pragma unroll
   for (int q = 0; q < NP; ++q) {
-    const L r = density_of<DEV>(rho_ref, f[q]);
+    const L r = density_of<DEV, EOS>(rho_ref, f[q]);
     C re[W];
 #pragma unroll
     for (int e = 0; e < W; ++e) re[e] = (fl[W * q + e] & FLAG_SOLID) ? C(1) : el(r, e);
@@ -534,7 +534,7 @@ __global__ void __launch_bounds__(VW* Vec<S>::VH, Vec<S>::kBlocks)
         }
         psi_s[LBM_CHK(prow, VH + 2)][LBM_CHK(pj(pcol), SWP)] = (nf & FLAG_SOLID)
                                 ? psi_w
-                                : psi_of<C, EOS>(k, density_of<DEV>(rho_ref, g));
+                                : psi_of<C, EOS>(k, density_of<DEV, EOS>(rho_ref, g));
       }
     }
     __syncthreads();  // psi_s complete

@@ -11,11 +11,6 @@ namespace wall {
 constexpr uint8_t kFromA = 1;   // X2 is read from lattice A (pre-collision)
 constexpr uint8_t kGhost = 2;   // the link has the ghost-node term chi f_eq(x_s)
 
-// a b + c: one rounding in FP64 (whose pipe is narrow), two in FP32, where it writes out what a plain
-// expression means without contraction.
-__device__ __forceinline__ double mad(double a, double b, double c) { return __fma_rn(a, b, c); }
-__device__ __forceinline__ float mad(float a, float b, float c) { return a * b + c; }
-
 // e_a . (x, y)
 template <typename T>
 __device__ __forceinline__ T edot(int a, T x, T y) {
@@ -27,8 +22,8 @@ __device__ __forceinline__ T edot(int a, T x, T y) {
 template <typename T>
 __device__ __forceinline__ T bracket(int a, T usx, T usy, T ubx, T uby) {
   const T eub = edot(a, ubx, uby);
-  const T t = mad(T(4.5) * eub, eub, mad(T(3), edot(a, usx, usy), T(1)));
-  return wgt<T>(a) * mad(T(-1.5), mad(ubx, ubx, uby * uby), t);
+  return wgt<T>(a) * (T(1) + T(3) * edot(a, usx, usy) + T(4.5) * eub * eub -
+                      T(1.5) * (ubx * ubx + uby * uby));
 }
 
 template <typename S>
@@ -148,9 +143,9 @@ __device__ __forceinline__ void fict_terms(int scheme, const Link<T>& q, const O
 template <typename T>
 __device__ __forceinline__ T link_value(const Link<T>& q, const Operands<T>& o, T rho_g) {
   T val = q.c0 * o.fo;
-  if (q.x1 >= 0) val = mad(q.c1, o.X1, val);
-  if (q.x2 >= 0) val = mad(q.c2, o.X2, val);
-  if (q.act && (q.kind & kGhost)) val = mad(q.chi, rho_g * o.br, val);
+  if (q.x1 >= 0) val += q.c1 * o.X1;
+  if (q.x2 >= 0) val += q.c2 * o.X2;
+  if (q.act && (q.kind & kGhost)) val += q.chi * (rho_g * o.br);
   return val;
 }
 

@@ -30,7 +30,7 @@ def _nvcc():
 
 
 def _sources():
-    names = CUDA_SOURCES + CXX_SOURCES + ["d2q9.cuh", "step_core.cuh", "wall.cuh", "wall_tile.cuh",
+    names = CUDA_SOURCES + CXX_SOURCES + ["d2q9.cuh", "step_core.cuh", "wall.cuh", "wall_tile.cuh", "wall_front.cuh",
                                            "tma.cuh", "lbm_internal.h"]
     paths = [os.path.join(CSRC, n) for n in names]
     paths.append(os.path.join(os.path.dirname(HERE), "include", "lbm_gb300.h"))
@@ -62,7 +62,8 @@ def build(force=False, verbose=False, checked=False):
         # inlined into the single-lattice and the batched wall kernels and the step kernels, and
         # must round identically in all of them so a lattice gives the same bits alone and in a
         # batch.  (The step kernels' own arithmetic is explicitly rounded.)
-        fmad = ["--fmad=false"] if src in ("boundary.cu", "step.cu") else []
+        fmad = ["--fmad=false"] if src in (
+            "boundary.cu", "step.cu", "step_vec.cu", "step_march.cu") else []
         cmd = [nvcc, *ARCH, "-O3", "-lineinfo", "-std=c++17", *fmad, *defs, "-Xcompiler", "-fPIC",
                "-Xcompiler", "-ffp-contract=off", "-c", os.path.join(CSRC, src), "-o", obj]
         procs.append((cmd, subprocess.Popen(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT)))

@@ -171,42 +171,6 @@ __global__ void tile_links_kernel(int n_nodes, const TileNode* __restrict__ node
   }
 }
 
-// The wall values written in place, into lattice B and the carry array.
-template <typename S>
-struct InPlace {
-  using T = typename Pop<S>::C;
-  void* f;
-  int N;
-  double* out;
-  __device__ __forceinline__ T incoming(int dst, int a, T v) const {
-    return Pop<S>::store_t(f, dst, N, v);
-  }
-  __device__ __forceinline__ T rest(int n, T v) const { return Pop<S>::store_t(f, n, N, v); }
-  __device__ __forceinline__ void carry(int b, double c) const { out[b] = c; }
-};
-
-// Channel ends (Sec. 4.2), after streaming and the wall pass; one thread per row j: the inlet at
-// i = 0, and at the outlet i = nx - 1 (fully developed flow) the populations entering from the right
-// (3, 6, 7) equal those of column nx - 2.
-template <typename S>
-__device__ __forceinline__ void open_row(const DevParams& p, int j, void* __restrict__ fb,
-                                         const uint8_t* __restrict__ flags, double u_in) {
-  const int nx = p.nx, N = p.N;
-  const bool in = j < p.ny;
-  const int n0 = in ? j * nx : 0, n1 = n0 + nx - 1;
-  const bool fluid0 = in && !(flags[n0] & FLAG_SOLID), fluid1 = in && !(flags[n1] & FLAG_SOLID);
-  pdl_wait();
-  if (fluid0)
-    inlet(p.rho_ref, u_in, [&](int a) { return Pop<S>::load_e(fb, a * N + n0, N); },
-          [&](int a, double v) { Pop<S>::store_e(fb, a * N + n0, N, v); });
-  if (fluid1) {
-    // copies of stored values: no rounding for any format
-    Pop<S>::store_e(fb, 3 * N + n1, N, Pop<S>::load_e(fb, 3 * N + n1 - 1, N));
-    Pop<S>::store_e(fb, 6 * N + n1, N, Pop<S>::load_e(fb, 6 * N + n1 - 1, N));
-    Pop<S>::store_e(fb, 7 * N + n1, N, Pop<S>::load_e(fb, 7 * N + n1 - 1, N));
-  }
-}
-
 // The wall pass: 8 lanes per boundary node.  CTAs from wall_ctas on (launched only in channel mode
 // when no boundary node reads or writes what the channel ends touch) do the channel ends, one
 // thread per row, so that the two need one launch.
@@ -221,7 +185,11 @@ __global__ void __launch_bounds__(128) boundary_kernel(DevParams p, int nb,
                                                        double* carry_out,
                                                        double* __restrict__ force, int wall_ctas,
                                                        const uint8_t* __restrict__ flags,
-                                                       double u_in) {
+                                                       double u_in, int* done) {
+  if (done && blockIdx.x == 0 && threadIdx.x < 2) {  // the counters of FrontWalls start at 0
+    pdl_wait();
+    done[threadIdx.x] = 0;
+  }
   if ((int)blockIdx.x >= wall_ctas) {
     open_row<S>(p, (blockIdx.x - wall_ctas) * blockDim.x + threadIdx.x, fb, flags, u_in);
     return;
@@ -286,14 +254,14 @@ cudaError_t launch_b(const DevParams& p, int nb, const int32_t* bnode, const int
                      const uint8_t* ldir, LinkRecipe r, const void* fa, void* fb,
                      const double* rho_m, const double* ux_m, const double* uy_m,
                      const double* carry_in, double* carry_out, double* force,
-                     const uint8_t* open_flags, double u_in, cudaStream_t s) {
+                     const uint8_t* open_flags, double u_in, int* done, cudaStream_t s) {
   const long long threads = 8LL * nb;
   const unsigned nt = wall_threads(threads + (open_flags ? p.ny : 0));
   const unsigned wall = (unsigned)((threads + nt - 1) / nt);
   const unsigned ends = open_flags ? (p.ny + nt - 1) / nt : 0;
   return launch_pdl(boundary_kernel<S>, dim3(wall + ends), dim3(nt), s, p, nb, bnode, boff, ldir,
                     r, fa, fb, rho_m, ux_m, uy_m, carry_in, carry_out, force, (int)wall, open_flags,
-                    u_in);
+                    u_in, done);
 }
 
 size_t align256(size_t v) { return (v + 255) / 256 * 256; }
@@ -391,16 +359,17 @@ cudaError_t launch_boundary(int precision, const DevParams& p, int nb, const int
                             const int32_t* boff, const uint8_t* ldir, LinkRecipe r,
                             const void* fa, void* fb, const double* rho_m, const double* ux_m,
                             const double* uy_m, const double* carry_in, double* carry_out,
-                            double* force, const uint8_t* open_flags, double u_in, cudaStream_t s) {
+                            double* force, const uint8_t* open_flags, double u_in, int* done,
+                            cudaStream_t s) {
   if (nb <= 0) return cudaSuccess;
   if (precision == LBM_FP32_DEV)
     return launch_b<float>(p, nb, bnode, boff, ldir, r, fa, fb, rho_m, ux_m, uy_m, carry_in, carry_out, force,
-                           open_flags, u_in, s);
+                           open_flags, u_in, done, s);
   if (precision == LBM_FP16_DEV)
     return launch_b<__half>(p, nb, bnode, boff, ldir, r, fa, fb, rho_m, ux_m, uy_m, carry_in, carry_out, force,
-                            open_flags, u_in, s);
+                            open_flags, u_in, done, s);
   return launch_b<double>(p, nb, bnode, boff, ldir, r, fa, fb, rho_m, ux_m, uy_m, carry_in, carry_out, force,
-                          open_flags, u_in, s);
+                          open_flags, u_in, done, s);
 }
 
 cudaError_t launch_open_x(int precision, const DevParams& p, void* fb, const uint8_t* flags,

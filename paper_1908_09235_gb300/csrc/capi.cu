@@ -88,15 +88,16 @@ cudaError_t launch_bulk(lbm_ctx* c, cudaStream_t s, int cur) {
 }
 
 // The wall pass and, in channel mode, the channel ends of a step from lattice cur; m: which set of
-// moments the step stored and which set of residues is current.  The new residues go to set 0.
-lbm_status launch_walls(lbm_ctx* c, cudaStream_t s, int cur, int m = 0) {
+// moments the step stored; r: which set of residues is current.  The new residues go to set 0.
+lbm_status launch_walls(lbm_ctx* c, cudaStream_t s, int cur, int m = 0, int r = 0) {
   void* fb = c->f[1 - cur];
   const bool together = c->open_x && c->ends_with_wall && c->nb > 0;
   cudaError_t e = launch_boundary(c->precision, c->p, (int)c->nb, c->bnode, c->boff, c->ldir,
                                   c->recipe, c->f[cur], fb, m ? c->macro2[0] : c->rho_m,
                                   m ? c->macro2[1] : c->ux_m, m ? c->macro2[2] : c->uy_m,
-                                  m ? c->carry2 : c->carry, c->carry, c->track_force ? c->force : nullptr,
-                                  together ? c->flags : nullptr, c->u_in, s);
+                                  r ? c->carry2 : c->carry, c->carry, c->track_force ? c->force : nullptr,
+                                  together ? c->flags : nullptr, c->u_in,
+                                  c->front ? c->front_done : nullptr, s);
   if (e != cudaSuccess) return cuda_fail(c, e, "boundary kernel launch");
   if (c->open_x && !together) {
     e = launch_open_x(c->precision, c->p, fb, c->flags, c->u_in, s);
@@ -114,14 +115,15 @@ lbm_status launch_one_step(lbm_ctx* c, cudaStream_t s, int cur) {
 // The wall pass of a step, and the channel ends where they touch other nodes, can be done by the next
 // step's kernel (but Zhao-Yong's wall pass reads the lattice which that kernel overwrites).
 bool walls_in_steps(const lbm_ctx* c) {
-  return c->tiles_shape >= 0 && c->nb > 0 && (!c->open_x || c->ends_with_wall) &&
+  const bool ends = c->ends_with_wall && (c->front || tiles_do_ends(c->tiles_shape));
+  return (c->tiles_shape >= 0 || c->front) && c->nb > 0 && (!c->open_x || ends) &&
          c->p.scheme != LBM_ZHAO_YONG;
 }
 
 // n steps from lattice cur, launched one after the other.  Where walls_in_steps, every kernel but
 // the first applies the wall pass of the step before it and only the last step's is a launch of its
-// own, so the lattice is complete between calls; the moments and residues a kernel reads were
-// stored in one set by the step before, its own go to the other.
+// own, so the lattice is complete between calls; the moments (and in the tiles the residues) a kernel
+// reads were stored in one set by the step before, its own go to the other.
 lbm_status launch_steps(lbm_ctx* c, cudaStream_t s, int cur, int n) {
   lbm_status st = LBM_OK;
   if (!walls_in_steps(c)) {
@@ -132,6 +134,26 @@ lbm_status launch_steps(lbm_ctx* c, cudaStream_t s, int cur, int n) {
   double* carry[2] = {c->carry, c->carry2};
   for (int k = 0; k < n; ++k, cur = 1 - cur) {
     const int m = k & 1;
+    if (c->front) {
+      cudaError_t e;
+      if (k == 0) {
+        e = launch_bulk(c, s, cur);
+      } else {
+        FrontWalls fw = c->fw;
+        fw.f = c->f[cur];
+        fw.rho = macro[1 - m][0];
+        fw.ux = macro[1 - m][1];
+        fw.uy = macro[1 - m][2];
+        fw.done = c->front_done + m;
+        fw.reset = c->front_done + 1 - m;
+        fw.open_x = c->open_x ? 1 : 0;
+        fw.u_in = c->u_in;
+        e = launch_step_front(c->precision, c->p, c->f[cur], c->f[1 - cur], c->flags, macro[m][0],
+                              macro[m][1], macro[m][2], fw, c->err_flag, s);
+      }
+      if (e != cudaSuccess) return cuda_fail(c, e, "step kernel launch");
+      continue;
+    }
     WallIn wi = c->tiles;
     wi.rho = macro[1 - m][0];
     wi.ux = macro[1 - m][1];
@@ -145,7 +167,8 @@ lbm_status launch_steps(lbm_ctx* c, cudaStream_t s, int cur, int n) {
                           macro[m][0], macro[m][1], macro[m][2], k > 0 ? &wi : nullptr, s);
     if (e != cudaSuccess) return cuda_fail(c, e, "step kernel launch");
   }
-  return n > 0 ? launch_walls(c, s, 1 - cur, (n - 1) & 1) : LBM_OK;
+  const int m = (n - 1) & 1;
+  return n > 0 ? launch_walls(c, s, 1 - cur, m, c->front ? 0 : m) : LBM_OK;
 }
 
 lbm_status build_graph(lbm_ctx* c, int parity) {
@@ -410,7 +433,7 @@ lbm_status lbm::create_context(const lbm_geometry* geo, const lbm_eos* eos, doub
   c->ends_with_wall = ends_clear_of_walls(g);
   size_t bytes = 2 * align_up(c->lattice_bytes) + align_up((N + 3) / 4 * 4) +
                  3 * align_up(N * 8) + align_up(c->ledger_blocks * 8) + align_up(8) +
-                 align_up(sizeof(int)) + align_up(gblocks * sizeof(int2)) + align_up(16);
+                 align_up(3 * sizeof(int)) + align_up(gblocks * sizeof(int2)) + align_up(16);
   void* base = dev_alloc(c, bytes);
   if (!base) {
     release_all(c);
@@ -426,7 +449,8 @@ lbm_status lbm::create_context(const lbm_geometry* geo, const lbm_eos* eos, doub
   c->uy_m = cv.take<double>(N);
   c->partials = cv.take<double>(c->ledger_blocks);
   c->mass_out = cv.take<double>(1);
-  c->err_flag = cv.take<int>(1);
+  c->err_flag = cv.take<int>(3);  // and FrontWalls' counters
+  c->front_done = c->err_flag + 1;
   c->geom_tmp = cv.take<int2>(gblocks);
   c->geom_totals = cv.take<long long>(2);
 
@@ -440,7 +464,7 @@ lbm_status lbm::create_context(const lbm_geometry* geo, const lbm_eos* eos, doub
   cudaError_t e;
   if ((e = cudaMemsetAsync(c->flags, 0, (N + 3) / 4 * 4, c->stream)) != cudaSuccess)
     return bail(e, "memset flags");
-  if ((e = cudaMemsetAsync(c->err_flag, 0, sizeof(int), c->stream)) != cudaSuccess)
+  if ((e = cudaMemsetAsync(c->err_flag, 0, 3 * sizeof(int), c->stream)) != cudaSuccess)
     return bail(e, "memset err");
   if ((e = launch_geom_solid(g, c->flags, c->stream)) != cudaSuccess) return bail(e, "geom solid");
   if ((e = launch_geom_count_scan(g, c->flags, c->geom_tmp, gblocks, c->geom_totals, c->stream)) !=
@@ -564,6 +588,30 @@ lbm_status lbm::create_context(const lbm_geometry* geo, const lbm_eos* eos, doub
     c->tiles.max_nodes = tt.max_nodes;
     c->tiles.cells = (tw + 2) * (th + 2);
     c->tiles_shape = fits ? shape : -1;
+  }
+  // ---- large lattices: the wall pass in front of the step kernel's tiles ----
+  if (!in_batch && shape < 0 && c->nb > 0 && !(opt && opt->kernel_path != 0) &&
+      step_front_supported(precision, eos->kind, geo->nx, geo->ny)) {
+    c->front = true;
+    for (int k = 0; k < 3; ++k) {
+      double* set0[3] = {c->rho_m, c->ux_m, c->uy_m};
+      c->macro2[k] = reinterpret_cast<double*>((float*)set0[k] + N);
+    }
+    FrontWalls& w = c->fw;
+    w.nb = (int)c->nb;
+    w.bnode = c->bnode;
+    w.boff = c->boff;
+    w.ldir = c->ldir;
+    w.recipe = c->recipe;
+    w.carry = c->carry;
+    w.flat = g.wall_q_lo > 0.0 || g.wall_q_hi > 0.0;
+    w.everywhere = g.n_circles > FrontWalls::kCircles;
+    w.n_circles = w.everywhere ? 0 : g.n_circles;
+    for (int k = 0; k < w.n_circles; ++k) {
+      w.cx[k] = (float)g.c[k].cx;
+      w.cy[k] = (float)g.c[k].cy;
+      w.r[k] = (float)g.c[k].r;
+    }
   }
   if ((e = cudaMemsetAsync(c->f[0], 0, c->lattice_bytes, c->stream)) != cudaSuccess)
     return bail(e, "memset f0");

@@ -74,6 +74,7 @@ struct GeomParams {
 
 struct LinkRecipe;
 struct WallIn;
+struct FrontWalls;
 
 // ---- launchers (implemented in the .cu files) ----
 // geometry.cu
@@ -98,7 +99,7 @@ bool step_vec_supported(int precision, int nx, int ny);
 cudaError_t launch_step_vec(int precision, const DevParams& p, const void* fa, void* fb,
                             const uint8_t* flags, double* rho_m, double* ux_m, double* uy_m,
                             bool fields_only, cudaStream_t s, bool tma_ring = false,
-                            int* err = nullptr);
+                            int* err = nullptr, const FrontWalls* front = nullptr);
 // path: 0 = for the deviation formats the marching kernel where step_march_supported(), the
 // vectorised kernel where step_vec_supported(), else the scalar tile kernel; 1 = the scalar tile kernel; 3 = the vectorised kernel where
 // step_vec_supported() (FP64 too), its psi ring staged by cp.async only; 4 = as 0.  Paths 0 and
@@ -111,12 +112,20 @@ cudaError_t launch_step(int precision, const DevParams& p, const void* fa, void*
 // kErrTimeout in *err.
 bool step_march_supported(int precision, int eos, int nx, int ny);
 cudaError_t launch_step_march(const DevParams& p, const void* fa, void* fb, const uint8_t* flags,
-                              double* rho_m, double* ux_m, double* uy_m, int* err, cudaStream_t s);
+                              double* rho_m, double* ux_m, double* uy_m, int* err, cudaStream_t s,
+                              const FrontWalls* front = nullptr);
+// The step with the front, by the marching kernel or (FP32 single phase) the vector kernel; front: its
+// rows and CTA counts are filled in here.
+bool step_front_supported(int precision, int eos, int nx, int ny);
+cudaError_t launch_step_front(int precision, const DevParams& p, const void* fa, void* fb,
+                              const uint8_t* flags, double* rho_m, double* ux_m, double* uy_m,
+                              FrontWalls front, int* err, cudaStream_t s);
 
 // The scalar tiles in the shapes of small lattices, whose step kernels can apply the previous
 // step's wall pass themselves (wi; nullptr: a plain step).  pick_step_tiles: the shape for a
 // lattice and its tile size, or -1 where the wall pass is a launch of its own.
 int pick_step_tiles(int precision, int eos, int nx, int ny, int* tw, int* th);
+bool tiles_do_ends(int shape);  // the shape's kernel does the channel ends too
 cudaError_t launch_step_tiles(int shape, int precision, const DevParams& p, const void* fa,
                               void* fb, const uint8_t* flags, double* rho_m, double* ux_m,
                               double* uy_m, const WallIn* wi, cudaStream_t s);
@@ -173,6 +182,26 @@ struct WallIn {
   double u_in;
 };
 
+// The wall pass of the step before and the channel ends as the first CTAs of a step kernel
+// (csrc/wall_front.cuh): they work on the kernel's source lattice f in place.
+struct FrontWalls {
+  int nb, wall_ctas, ctas, rows;  // boundary nodes; CTAs of the pass, with the ends; block rows they take
+  const int32_t* bnode;
+  const int32_t* boff;
+  const uint8_t* ldir;
+  LinkRecipe recipe;
+  void* f;
+  const double *rho, *ux, *uy;  // the moments that the step before stored
+  double* carry;
+  int *done, *reset;  // counts the front's CTAs in this step; the next step's counter
+  // the boundary nodes: near these circles, near the rows 0 and ny - 1 (flat), or anywhere
+  static constexpr int kCircles = 4;
+  int n_circles, flat, everywhere;
+  float cx[kCircles], cy[kCircles], r[kCircles];
+  int open_x;
+  double u_in;
+};
+
 // One lattice of a batch as the batched kernels see it.  cur and steps_left are advanced on
 // the device after every step (batch_advance_kernel), so a captured graph stays valid while
 // lattices join and leave the batch.
@@ -201,9 +230,11 @@ cudaError_t launch_boundary(int precision, const DevParams& p, int nb, const int
                             const int32_t* boff, const uint8_t* ldir, LinkRecipe r,
                             const void* fa, void* fb, const double* rho_m, const double* ux_m,
                             const double* uy_m, const double* carry_in, double* carry_out,
-                            double* force, const uint8_t* open_flags, double u_in, cudaStream_t s);
+                            double* force, const uint8_t* open_flags, double u_in, int* done,
+                            cudaStream_t s);
 // open_flags (with nb > 0): the node flags, to do the channel ends in the same launch (only where
-// they and the wall pass touch different nodes), or nullptr.  force: per boundary node (fx, fy) of the momentum exchange with the walls, or nullptr
+// they and the wall pass touch different nodes), or nullptr.  done: FrontWalls' two counters, to be
+// zeroed, or nullptr.  force: per boundary node (fx, fy) of the momentum exchange with the walls, or nullptr
 // Channel ends (velocity inlet at column 0, fully developed outlet at column nx - 1)
 cudaError_t launch_open_x(int precision, const DevParams& p, void* fb, const uint8_t* flags,
                           double u_in, cudaStream_t s);
@@ -302,6 +333,9 @@ struct lbm_ctx {
   // and the second set of moments and residues that alternate with the first from step to step
   int tiles_shape = -1;
   lbm::WallIn tiles{};
+  bool front = false;        // large lattices: the wall pass in front of the step kernel's tiles
+  lbm::FrontWalls fw{};      // its fixed part
+  int* front_done = nullptr;  // its two counters
   double* macro2[3] = {nullptr, nullptr, nullptr};
   double* carry2 = nullptr;
   double* force = nullptr;    // per boundary node (fx, fy) of the last step's momentum exchange

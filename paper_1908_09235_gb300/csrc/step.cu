@@ -289,6 +289,8 @@ int pick_step_tiles(int precision, int eos, int nx, int ny, int* tw, int* th) {
   return shape;
 }
 
+bool tiles_do_ends(int shape) { return shape >= 0 && kShapes[shape].mode == 1; }
+
 cudaError_t launch_step_tiles(int shape, int precision, const DevParams& p, const void* fa,
                               void* fb, const uint8_t* flags, double* rho_m, double* ux_m,
                               double* uy_m, const WallIn* wi, cudaStream_t s) {
@@ -297,6 +299,21 @@ cudaError_t launch_step_tiles(int shape, int precision, const DevParams& p, cons
   if (precision == LBM_FP16_DEV)
     return launch_tiles_s<__half>(shape, p, fa, fb, flags, rho_m, ux_m, uy_m, wi, s);
   return launch_tiles_s<double>(shape, p, fa, fb, flags, rho_m, ux_m, uy_m, wi, s);
+}
+
+bool step_front_supported(int precision, int eos, int nx, int ny) {
+  return step_march_supported(precision, eos, nx, ny) ||
+         (precision == LBM_FP32_DEV && eos == LBM_EOS_NONE &&
+          step_vec_supported(precision, nx, ny));
+}
+
+cudaError_t launch_step_front(int precision, const DevParams& p, const void* fa, void* fb,
+                              const uint8_t* flags, double* rho_m, double* ux_m, double* uy_m,
+                              FrontWalls front, int* err, cudaStream_t s) {
+  if (step_march_supported(precision, p.eos, p.nx, p.ny))
+    return launch_step_march(p, fa, fb, flags, rho_m, ux_m, uy_m, err, s, &front);
+  return launch_step_vec(precision, p, fa, fb, flags, rho_m, ux_m, uy_m, false, s, true, err,
+                         &front);
 }
 
 cudaError_t launch_step(int precision, const DevParams& p, const void* fa, void* fb,

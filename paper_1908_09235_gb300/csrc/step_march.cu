@@ -18,6 +18,7 @@
 // not the instruction cache: 184.  FP32 deviations the same way: 201-220 against 195 us, so not theirs.
 #include "step_core.cuh"
 #include "tma.cuh"
+#include "wall_front.cuh"
 
 namespace lbm {
 
@@ -71,13 +72,15 @@ __device__ __forceinline__ void store1(void* b, int a, int N, int n, float v) {
   *moving_at(b, a, N, LBM_CHK(n, N)) = __float2half_rn(v);
 }
 
-template <int EOS>
+// FRONT: the first block rows are the wall pass of the step before (csrc/wall_front.cuh).
+template <int EOS, bool FRONT>
 __global__ void __launch_bounds__(32, kWarps)
-    step_march_kernel(DevParams p, const void* __restrict__ fa, void* __restrict__ fb,
+    step_march_kernel(const __grid_constant__ DevParams p, const void* fa, void* __restrict__ fb,
                       const uint8_t* __restrict__ flags, float* __restrict__ rho_m,
                       float* __restrict__ ux_m, float* __restrict__ uy_m,
                       const __grid_constant__ CUtensorMap map,
-                      const __grid_constant__ CUtensorMap map2, int* __restrict__ err) {
+                      const __grid_constant__ CUtensorMap map2, int* __restrict__ err,
+                      const __grid_constant__ FrontWalls front) {
   using S = __half;
   using L = float2;
   constexpr int R = kSlots;
@@ -87,10 +90,19 @@ __global__ void __launch_bounds__(32, kWarps)
   const int nx = p.nx, ny = p.ny, N = p.N;
   const Consts<float>& k = p.cf;
   const float rho_ref = k.rho_ref, psi_w = k.psi_wall;
+  int by = blockIdx.y, strips = gridDim.y;
+  if constexpr (FRONT) {
+    if (by < front.rows) {
+      wall::front_cta<S>(p, front, flags, by * gridDim.x + blockIdx.x, lane, 32);
+      return;
+    }
+    by -= front.rows;
+    strips -= front.rows;
+  }
   const int x0 = blockIdx.x * SWD;
   // rows y0 .. y1 - 1 (the strips' heights differ by one at most)
-  const int y0 = (int)((long long)blockIdx.y * ny / gridDim.y);
-  const int y1 = (int)((long long)(blockIdx.y + 1) * ny / gridDim.y);
+  const int y0 = (int)((long long)by * ny / strips);
+  const int y1 = (int)((long long)(by + 1) * ny / strips);
   const int nv = min(32, (nx - x0) >> 2);  // lanes with nodes inside the lattice
   const bool lane_ok = lane < nv, first = lane == 0, last = lane == nv - 1;
   const int col = x0 + 4 * (lane_ok ? lane : 0);
@@ -108,6 +120,12 @@ __global__ void __launch_bounds__(32, kWarps)
   };
   uint32_t fl_c = row_flags(y0 - 1), fl_n = row_flags(y0);
   pdl_wait();
+  if constexpr (FRONT) {
+    if (wall::front_touches(front, x0, y0, SWD, y1 - y0, nx, ny)) {
+      if (lane == 0) wall::front_wait(front, err);
+      __syncwarp();
+    }
+  }
   // row y goes to slot (y - y0 + 1) % R
   auto fetch = [&](int y, int s) {
     if (lane == 0) {
@@ -280,13 +298,21 @@ __global__ void __launch_bounds__(32, kWarps)
 
 template <int EOS>
 cudaError_t launch_march_t(const DevParams& p, const void* fa, void* fb, const uint8_t* flags,
-                           double* rho_m, double* ux_m, double* uy_m, int* err, cudaStream_t s) {
+                           double* rho_m, double* ux_m, double* uy_m, int* err, cudaStream_t s,
+                           const FrontWalls* front) {
   CUtensorMap map{}, map2{};
   if (!make_ring_tensor_maps_fp16(&map, &map2, fa, p.nx, p.ny, SWD, SWD))
     return cudaErrorNotSupported;
-  const dim3 grid((p.nx + SWD - 1) / SWD, (p.ny + kRows - 1) / kRows);
-  return launch_pdl(step_march_kernel<EOS>, grid, dim3(32), s, p, fa, fb, flags, (float*)rho_m,
-                    (float*)ux_m, (float*)uy_m, map, map2, err);
+  dim3 grid((p.nx + SWD - 1) / SWD, (p.ny + kRows - 1) / kRows);
+  if (!front)
+    return launch_pdl(step_march_kernel<EOS, false>, grid, dim3(32), s, p, fa, fb, flags,
+                      (float*)rho_m, (float*)ux_m, (float*)uy_m, map, map2, err, FrontWalls{});
+  FrontWalls w = *front;
+  w.wall_ctas = w.ctas = (8 * w.nb + 31) / 32;
+  w.rows = (w.ctas + grid.x - 1) / grid.x;
+  grid.y += w.rows;
+  return launch_pdl(step_march_kernel<EOS, true>, grid, dim3(32), s, p, fa, fb, flags,
+                    (float*)rho_m, (float*)ux_m, (float*)uy_m, map, map2, err, w);
 }
 
 }  // namespace
@@ -299,11 +325,11 @@ bool step_march_supported(int precision, int eos, int nx, int ny) {
 }
 
 cudaError_t launch_step_march(const DevParams& p, const void* fa, void* fb, const uint8_t* flags,
-                              double* rho_m, double* ux_m, double* uy_m, int* err,
-                              cudaStream_t s) {
+                              double* rho_m, double* ux_m, double* uy_m, int* err, cudaStream_t s,
+                              const FrontWalls* front) {
   if (p.eos == LBM_EOS_EXP)
-    return launch_march_t<LBM_EOS_EXP>(p, fa, fb, flags, rho_m, ux_m, uy_m, err, s);
-  return launch_march_t<LBM_EOS_CS>(p, fa, fb, flags, rho_m, ux_m, uy_m, err, s);
+    return launch_march_t<LBM_EOS_EXP>(p, fa, fb, flags, rho_m, ux_m, uy_m, err, s, front);
+  return launch_march_t<LBM_EOS_CS>(p, fa, fb, flags, rho_m, ux_m, uy_m, err, s, front);
 }
 
 }  // namespace lbm

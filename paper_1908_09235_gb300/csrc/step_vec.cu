@@ -31,6 +31,7 @@
 
 #include "step_core.cuh"
 #include "tma.cuh"
+#include "wall_front.cuh"
 
 namespace lbm {
 
@@ -255,9 +256,13 @@ __device__ __forceinline__ void load_flags(const uint8_t* flags, int n, uint8_t 
 // per row (rmap, box SWE x 1 x 9); FP16 two (rmap: the FP32 rest plane, box SWE x 1; rmap2: the
 // eight FP16 planes, box kTmaWidth x 1 x 8).  Their wait is bounded (an expired wait sets
 // kErrTimeout in *err).
-template <typename S, int EOS, bool FIELDS, bool TR>
+// FRONT (single phase): the first block rows are the wall pass of the step before
+// (csrc/wall_front.cuh).  FP32 us a step at 1600 x 1000 / 2048^2 / 4096^2: 17.8 / 47.2 / 179.4 against
+// 19.3 / 50.1 / 182.2 with the pass apart.  Not for psi, where the same slowed the tiles by more than
+// the pass costs (4096^2 FP32 212 against 200), nor FP16 (single phase 134.6 against 123.3).
+template <typename S, int EOS, bool FIELDS, bool TR, bool FRONT>
 __global__ void __launch_bounds__(VW* Vec<S>::VH, Vec<S>::kBlocks)
-    step_vec_kernel(DevParams p, const void* __restrict__ fa, void* __restrict__ fb,
+    step_vec_kernel(const __grid_constant__ DevParams p, const void* fa, void* __restrict__ fb,
                     const uint8_t* __restrict__ flags, double* __restrict__ rho_m,
                     double* __restrict__ ux_m, double* __restrict__ uy_m,
                     const __grid_constant__ CUtensorMap rmap,
@@ -265,7 +270,7 @@ __global__ void __launch_bounds__(VW* Vec<S>::VH, Vec<S>::kBlocks)
                     const __grid_constant__ CUtensorMap pmap,
                     const __grid_constant__ CUtensorMap pmap2,
                     const __grid_constant__ CUtensorMap fmap, int pf_flags,
-                    int* __restrict__ err) {
+                    int* __restrict__ err, const __grid_constant__ FrontWalls front) {
   using C = typename Pop<S>::C;
   using VT = Vec<S>;
   constexpr int V = VT::V;
@@ -290,12 +295,21 @@ __global__ void __launch_bounds__(VW* Vec<S>::VH, Vec<S>::kBlocks)
 
   const int lane = threadIdx.x, w = threadIdx.y, tid = w * VW + lane;
   const int nx = p.nx, ny = p.ny, N = p.N;
-  const int x0 = blockIdx.x * TW, y0 = blockIdx.y * VH;
+  int rows = 0;  // block rows before the first tile
+  if constexpr (FRONT) {
+    rows = front.rows;
+    if ((int)blockIdx.y < rows) {
+      wall::front_cta<S>(p, front, flags, blockIdx.y * gridDim.x + blockIdx.x, tid, VW * VH);
+      return;
+    }
+  }
+  const int by = blockIdx.y - rows;
+  const int x0 = blockIdx.x * TW, y0 = by * VH;
   if constexpr (TR && PSI && (VT::kPrefetchPops || VT::kPrefetchFlags)) {
     // the populations and flags of the tile kPrefetchAhead CTAs later in launch order go to L2
     // now, by tensor-copy prefetches of one tile-sized box each, so that its loads find them there
-    const int t = blockIdx.y * gridDim.x + blockIdx.x + VT::kPrefetchAhead;
-    if (tid == 32 && t < gridDim.x * gridDim.y) {
+    const int t = by * gridDim.x + blockIdx.x + VT::kPrefetchAhead;
+    if (tid == 32 && t < (int)(gridDim.x * (gridDim.y - rows))) {
       const int px = (t % gridDim.x) * TW, py = (t / gridDim.x) * VH;
       if constexpr (VT::kPrefetchPops) {
         if constexpr (sizeof(S) == 2) {
@@ -469,6 +483,31 @@ __global__ void __launch_bounds__(VW* Vec<S>::VH, Vec<S>::kBlocks)
     issue_ring_copies();
     load_flags<V>(flags, LBM_CHK(n, N - V + 1), fl);
     load_own();
+  }
+
+  // Nodes that the front writes (boundary nodes, and with open ends the columns 0 and nx - 1) are read
+  // again once it is done, by the lanes that have one; the flags, awaited anyway, tell them.
+  if constexpr (FRONT) {
+    bool again[V], any = false;
+#pragma unroll
+    for (int v = 0; v < V; ++v) {
+      const int x = x0 + V * lane + v;
+      again[v] = lane_ok && ((fl[v] & FLAG_BOUNDARY) || (front.open_x && !(fl[v] & FLAG_SOLID) &&
+                                                         (x == 0 || x == nx - 1)));
+      any = any || again[v];
+    }
+    if (any) {
+      wall::front_wait(front, err);
+#pragma unroll
+      for (int v = 0; v < V; ++v)
+        if (again[v]) {
+#pragma unroll
+          for (int a = 0; a < 9; ++a) {
+            const C t = Pop<S>::load(fa, a, N, n + v);
+            if constexpr (W == 2) (v & 1 ? f[v >> 1][a].y : f[v >> 1][a].x) = t; else f[v][a] = t;
+          }
+        }
+    }
   }
 
   L rho[NP], inv[NP];
@@ -653,19 +692,18 @@ __global__ void __launch_bounds__(VW* Vec<S>::VH, Vec<S>::kBlocks)
   }
 }
 
-template <typename S, int EOS>
-cudaError_t launch_vec_t(const DevParams& p, const void* fa, void* fb, const uint8_t* flags,
-                         double* rho_m, double* ux_m, double* uy_m, bool fields_only,
-                         cudaStream_t s, bool tma_ring, int* err) {
+template <typename S, int EOS, bool FRONT>
+cudaError_t launch_vec_f(const DevParams& p, const void* fa, void* fb, const uint8_t* flags,
+                         double* rho_m, double* ux_m, double* uy_m, cudaStream_t s, bool tma_ring,
+                         int* err, const FrontWalls& front) {
   constexpr int TW = VW * Vec<S>::V, VH = Vec<S>::VH;
-  dim3 block(VW, VH);
-  dim3 grid((p.nx + TW - 1) / TW, (p.ny + VH - 1) / VH);
+  const dim3 block(VW, VH), grid((p.nx + TW - 1) / TW, (p.ny + VH - 1) / VH + front.rows);
   // ring-row and tile-prefetch maps; unused by the kernels without tensor copies
   CUtensorMap map{}, map2{}, pmap{}, pmap2{}, fmap{};
   int pf_flags = 0;  // fmap valid (row pitch of the flags a multiple of 16 bytes)
   if constexpr (!std::is_same<S, double>::value && EOS != LBM_EOS_NONE) {
     constexpr bool fp16 = std::is_same<S, __half>::value;
-    bool maps = tma_ring && !fields_only && err;
+    bool maps = tma_ring && err;
     if (maps) {
       if constexpr (fp16)
         maps = make_ring_tensor_maps_fp16(&map, &map2, fa, p.nx, p.ny, Vec<S>::SWE,
@@ -677,34 +715,56 @@ cudaError_t launch_vec_t(const DevParams& p, const void* fa, void* fb, const uin
       if (maps && Vec<S>::kPrefetchFlags)
         pf_flags = make_flags_prefetch_map(&fmap, flags, p.nx, p.ny, TW, VH) ? 1 : 0;
     }
-    if (maps) {
-      return launch_pdl(step_vec_kernel<S, EOS, false, true>, grid, block, s, p, fa, fb, flags,
-                        rho_m, ux_m, uy_m, map, map2, pmap, pmap2, fmap, pf_flags, err);
-    }
+    if (maps)
+      return launch_pdl(step_vec_kernel<S, EOS, false, true, FRONT>, grid, block, s, p, fa, fb,
+                        flags, rho_m, ux_m, uy_m, map, map2, pmap, pmap2, fmap, pf_flags, err,
+                        front);
   }
+  return launch_pdl(step_vec_kernel<S, EOS, false, false, FRONT>, grid, block, s, p, fa, fb, flags,
+                    rho_m, ux_m, uy_m, map, map2, pmap, pmap2, fmap, 0, err, front);
+}
+
+template <typename S, int EOS>
+cudaError_t launch_vec_t(const DevParams& p, const void* fa, void* fb, const uint8_t* flags,
+                         double* rho_m, double* ux_m, double* uy_m, bool fields_only,
+                         cudaStream_t s, bool tma_ring, int* err, const FrontWalls* front) {
   if (fields_only) {
-    step_vec_kernel<S, EOS, true, false><<<grid, block, 0, s>>>(
-        p, fa, fb, flags, rho_m, ux_m, uy_m, map, map2, pmap, pmap2, fmap, 0, err);
+    constexpr int TW = VW * Vec<S>::V, VH = Vec<S>::VH;
+    const dim3 block(VW, VH), grid((p.nx + TW - 1) / TW, (p.ny + VH - 1) / VH);
+    const CUtensorMap none{};
+    step_vec_kernel<S, EOS, true, false, false><<<grid, block, 0, s>>>(
+        p, fa, fb, flags, rho_m, ux_m, uy_m, none, none, none, none, none, 0, err, FrontWalls{});
     return cudaGetLastError();
   }
-  return launch_pdl(step_vec_kernel<S, EOS, false, false>, grid, block, s, p, fa, fb, flags, rho_m,
-                    ux_m, uy_m, map, map2, pmap, pmap2, fmap, 0, err);
+  if constexpr (std::is_same<S, float>::value && EOS == LBM_EOS_NONE) {
+    if (front) {
+      FrontWalls w = *front;
+      constexpr int NT = VW * Vec<S>::VH;
+      w.wall_ctas = (8 * w.nb + NT - 1) / NT;
+      w.ctas = w.wall_ctas + (w.open_x ? (p.ny + NT - 1) / NT : 0);
+      const int tx = (p.nx + VW * Vec<S>::V - 1) / (VW * Vec<S>::V);
+      w.rows = (w.ctas + tx - 1) / tx;
+      return launch_vec_f<S, EOS, true>(p, fa, fb, flags, rho_m, ux_m, uy_m, s, tma_ring, err, w);
+    }
+  }
+  return launch_vec_f<S, EOS, false>(p, fa, fb, flags, rho_m, ux_m, uy_m, s, tma_ring, err,
+                                     FrontWalls{});
 }
 
 template <typename S>
 cudaError_t launch_vec_s(const DevParams& p, const void* fa, void* fb, const uint8_t* flags,
                          double* rho_m, double* ux_m, double* uy_m, bool fields_only,
-                         cudaStream_t s, bool tma_ring, int* err) {
+                         cudaStream_t s, bool tma_ring, int* err, const FrontWalls* front) {
   switch (p.eos) {
     case LBM_EOS_EXP:
       return launch_vec_t<S, LBM_EOS_EXP>(p, fa, fb, flags, rho_m, ux_m, uy_m, fields_only, s,
-                                          tma_ring, err);
+                                          tma_ring, err, front);
     case LBM_EOS_CS:
       return launch_vec_t<S, LBM_EOS_CS>(p, fa, fb, flags, rho_m, ux_m, uy_m, fields_only, s,
-                                         tma_ring, err);
+                                         tma_ring, err, front);
     default:
       return launch_vec_t<S, LBM_EOS_NONE>(p, fa, fb, flags, rho_m, ux_m, uy_m, fields_only, s,
-                                           tma_ring, err);
+                                           tma_ring, err, front);
   }
 }
 
@@ -721,14 +781,16 @@ bool step_vec_supported(int precision, int nx, int ny) {
 
 cudaError_t launch_step_vec(int precision, const DevParams& p, const void* fa, void* fb,
                             const uint8_t* flags, double* rho_m, double* ux_m, double* uy_m,
-                            bool fields_only, cudaStream_t s, bool tma_ring, int* err) {
+                            bool fields_only, cudaStream_t s, bool tma_ring, int* err,
+                            const FrontWalls* front) {
   if (precision == LBM_FP32_DEV)
     return launch_vec_s<float>(p, fa, fb, flags, rho_m, ux_m, uy_m, fields_only, s, tma_ring,
-                               err);
+                               err, front);
   if (precision == LBM_FP16_DEV)
     return launch_vec_s<__half>(p, fa, fb, flags, rho_m, ux_m, uy_m, fields_only, s, tma_ring,
-                                err);
-  return launch_vec_s<double>(p, fa, fb, flags, rho_m, ux_m, uy_m, fields_only, s, false, err);
+                                err, front);
+  return launch_vec_s<double>(p, fa, fb, flags, rho_m, ux_m, uy_m, fields_only, s, false, err,
+                              nullptr);
 }
 
 }  // namespace lbm

@@ -267,5 +267,41 @@ __device__ __forceinline__ void wall_values(const DevParams& p, int b, int k, bo
   }
 }
 
+// The wall values written in place, into lattice B and the carry array.
+template <typename S>
+struct InPlace {
+  using T = typename Pop<S>::C;
+  void* f;
+  int N;
+  double* out;
+  __device__ __forceinline__ T incoming(int dst, int a, T v) const {
+    return Pop<S>::store_t(f, dst, N, v);
+  }
+  __device__ __forceinline__ T rest(int n, T v) const { return Pop<S>::store_t(f, n, N, v); }
+  __device__ __forceinline__ void carry(int b, double c) const { out[b] = c; }
+};
+
+// Channel ends (Sec. 4.2), after streaming and the wall pass; one thread per row j: the inlet at
+// i = 0, and at the outlet i = nx - 1 (fully developed flow) the populations entering from the right
+// (3, 6, 7) equal those of column nx - 2.
+template <typename S>
+__device__ __forceinline__ void open_row(const DevParams& p, int j, void* __restrict__ fb,
+                                         const uint8_t* __restrict__ flags, double u_in) {
+  const int nx = p.nx, N = p.N;
+  const bool in = j < p.ny;
+  const int n0 = in ? j * nx : 0, n1 = n0 + nx - 1;
+  const bool fluid0 = in && !(flags[n0] & FLAG_SOLID), fluid1 = in && !(flags[n1] & FLAG_SOLID);
+  pdl_wait();
+  if (fluid0)
+    inlet(p.rho_ref, u_in, [&](int a) { return Pop<S>::load_e(fb, a * N + n0, N); },
+          [&](int a, double v) { Pop<S>::store_e(fb, a * N + n0, N, v); });
+  if (fluid1) {
+    // copies of stored values: no rounding for any format
+    Pop<S>::store_e(fb, 3 * N + n1, N, Pop<S>::load_e(fb, 3 * N + n1 - 1, N));
+    Pop<S>::store_e(fb, 6 * N + n1, N, Pop<S>::load_e(fb, 6 * N + n1 - 1, N));
+    Pop<S>::store_e(fb, 7 * N + n1, N, Pop<S>::load_e(fb, 7 * N + n1 - 1, N));
+  }
+}
+
 }  // namespace wall
 }  // namespace lbm

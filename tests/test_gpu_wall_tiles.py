@@ -91,6 +91,24 @@ def test_every_tile_shape_gives_the_bits_of_the_wall_kernel(gpu_lib, precision, 
                      _run([35], *args, 1, kind, circles, False)), scheme
 
 
+@pytest.mark.parametrize("precision,nx,ny,kind", [
+    (lbm.FP32_DEV, 1600, 1603, "cs"), (lbm.FP16_DEV, 1124, 1125, "exp"),
+    (lbm.FP16_DEV, 1128, 1125, "cs"), (lbm.FP32_DEV, 700, 610, "none"),
+    (lbm.FP16_DEV, 644, 509, "none"), (lbm.FP32_DEV, 2056, 1250, "exp"),
+])
+def test_walls_in_front_of_the_tiles_give_the_bits_of_the_wall_kernel(gpu_lib, precision, nx, ny,
+                                                                      kind):
+    # large lattices (vector and marching kernel): ragged tiles in x and y, walls along the seam, two
+    # bodies, one of them on tile edges; kernel_path 4 is the same kernel with the wall pass apart
+    circles = [(0.3 * nx, 0.35 * ny, 0.11 * nx), (640.0 if nx > 700 else 512.0, 0.3 * ny, 20.5)]
+    for scheme in ("bouzidi_q", "mod_a", "mod_b"):
+        for walls in (False, True):
+            args = (nx, ny, precision, scheme)
+            apart = _run([5], *args, 4, kind, circles, walls)
+            assert _same(_run([5], *args, 0, kind, circles, walls), apart), (scheme, walls)
+            assert _same(_run([2, 1, 2], *args, 0, kind, circles, walls), apart), (scheme, walls)
+
+
 @pytest.mark.parametrize("precision", [lbm.FP64, lbm.FP32_DEV, lbm.FP16_DEV])
 @pytest.mark.parametrize("nx,ny", [(120, 64), (121, 75), (800, 500)])
 def test_channel_ends_in_the_tiles_give_the_bits_of_their_kernel(gpu_lib, precision, nx, ny):

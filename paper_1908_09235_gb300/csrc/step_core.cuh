@@ -388,18 +388,47 @@ __device__ __forceinline__ void step_tile(const DevParams& p, const void* __rest
         if ((fl[r] & (FLAG_SOLID | FLAG_BOUNDARY)) == FLAG_BOUNDARY &&
             (EOS != LBM_EOS_NONE || (x < nx && y0 + ty + r * TYN < ny)))
           walls.take(p, (ty + r * TYN + 1) * (TXN + 2) + tx + 1, f[r]);
-      // (the inlet's FP64 arithmetic only where registers are plenty: inline in WALL 2 it made a
-      // 1241 x 775 channel 23.3 us a step, 21.7 with the ends apart before)
+      // Channel ends.  (The inlet's FP64 arithmetic only where registers are plenty: inline in WALL 2
+      // it made a 1241 x 775 channel 23.3 us a step, 21.7 with the ends apart before.)  The tile's
+      // rows go through one warp, one per lane: in the lanes of column 0 every warp of the tile
+      // would take its turn on the narrow FP64 pipe.
       if constexpr (EOS == LBM_EOS_NONE && WALL == 1) {
-        if (wi->open_x && (x == 0 || x == nx - 1)) {
+        __shared__ C ends_s[TH][6];
+        constexpr int known[6] = {0, 2, 3, 4, 6, 7};
+        if (wi->open_x && x0 == 0) {
+          if (x == 0) {
+#pragma unroll
+            for (int r = 0; r < RY; ++r)
+#pragma unroll
+              for (int i = 0; i < 6; ++i) ends_s[ty + r * TYN][i] = f[r][known[i]];
+          }
+          __syncthreads();
+          if (c < TH) {
+            C g[9];
+#pragma unroll
+            for (int i = 0; i < 6; ++i) g[known[i]] = ends_s[c][i];
+            wall::inlet(p.rho_ref, wi->u_in, [&](int a) { return double(g[a]); },
+                        [&](int a, double v) { g[a] = Pop<S>::rounded_e(a, v); });
+            ends_s[c][0] = g[1];
+            ends_s[c][1] = g[5];
+            ends_s[c][2] = g[8];
+          }
+          __syncthreads();
+          if (x == 0) {
+#pragma unroll
+            for (int r = 0; r < RY; ++r) {
+              if (fl[r] & FLAG_SOLID) continue;
+              f[r][1] = ends_s[ty + r * TYN][0];
+              f[r][5] = ends_s[ty + r * TYN][1];
+              f[r][8] = ends_s[ty + r * TYN][2];
+            }
+          }
+        }
+        if (wi->open_x && x == nx - 1) {
 #pragma unroll
           for (int r = 0; r < RY; ++r) {
             if (fl[r] & FLAG_SOLID) continue;
-            if (x == 0)
-              wall::inlet(p.rho_ref, wi->u_in, [&](int a) { return double(f[r][a]); },
-                          [&](int a, double v) { f[r][a] = Pop<S>::rounded_e(a, v); });
-            else
-              for (int a : {3, 6, 7}) f[r][a] = Pop<S>::load(fa, a, N, own_node(r) - 1);
+            for (int a : {3, 6, 7}) f[r][a] = Pop<S>::load(fa, a, N, own_node(r) - 1);
           }
         }
       }

@@ -30,7 +30,7 @@ SCHEME_NAMES = ("mls", "bouzidi_l", "zhao_yong", "mod_a", "mod_b")
 # FP64 pipe operations (DFMA + DADD + DMUL thread instructions) per fluid-node update of the FP64
 # step kernel, counted by ncu on the 2048^2 case (profiles/step_kernel_fp64_4096.md): with the
 # measured FMA rate of the pipe it gives the FP64 step's ALU roofline
-FP64_PIPE_OPS_PER_NODE = 128
+FP64_PIPE_OPS_PER_NODE = 113
 
 
 def bytes_per_update(precision):

@@ -142,7 +142,8 @@ typedef struct {
                         * 3: the vectorised kernel wherever nx % 4 == 0 (FP64: nx % 2 == 0) and *
                         *    ny >= 8 (FP16: 12), FP64 included, its halo staged by cp.async     *
                         *    only; otherwise the scalar tiles;                                   *
-                        * 4: the same as 0                                                       */
+                        * 4: the kernels of 0 for large lattices at every size, the wall pass    *
+                        *    always a launch of its own                                          */
   int32_t track_force; /* nonzero: the wall pass records the momentum exchange for lbm_force   *
                         * (also switched on by lbm_set_inflow); off by default, it costs the   *
                         * wall pass a few microseconds per step; ignored by batches            */

@@ -190,6 +190,11 @@ lbm_status build_graph(lbm_ctx* c, int parity) {
 
 bool is_fin(double v) { return std::isfinite(v); }
 
+bool crosses_seam(const lbm_circle& c, int nx, int ny) {  // or comes within two nodes of it
+  return c.cx - c.r - 2 < 0 || c.cx + c.r + 2 > nx - 1 || c.cy - c.r - 2 < 0 ||
+         c.cy + c.r + 2 > ny - 1;
+}
+
 // The wall pass and the channel ends touch different nodes: every solid body is a disc, so the
 // wall pass reads and writes nodes within its box widened by 1 + 2 (a boundary node, and two
 // nodes behind it); the ends touch columns 0, nx - 2 and nx - 1.
@@ -344,9 +349,7 @@ lbm_status lbm::create_context(const lbm_geometry* geo, const lbm_eos* eos, doub
   for (int k = 0; k < geo->n_circles; ++k) {
     const lbm_circle& cc = geo->circles[k];
     if (!(cc.r > 0) || !is_fin(cc.cx) || !is_fin(cc.cy) || !is_fin(cc.r)) return LBM_EINVAL;
-    if (cc.cx - cc.r - 2 < 0 || cc.cx + cc.r + 2 > geo->nx - 1 || cc.cy - cc.r - 2 < 0 ||
-        cc.cy + cc.r + 2 > geo->ny - 1)
-      if (!cc.solid_outside) return LBM_EINVAL;  // would cross the periodic seam
+    if (!cc.solid_outside && crosses_seam(cc, geo->nx, geo->ny)) return LBM_EINVAL;
   }
   if (!(geo->wall_q_lo <= 1.0) || !(geo->wall_q_hi <= 1.0)) return LBM_EINVAL;
 
@@ -605,7 +608,10 @@ lbm_status lbm::create_context(const lbm_geometry* geo, const lbm_eos* eos, doub
     w.recipe = c->recipe;
     w.carry = c->carry;
     w.flat = g.wall_q_lo > 0.0 || g.wall_q_hi > 0.0;
+    // (a circle round the fluid may cross the seam, and then has boundary nodes all along it)
     w.everywhere = g.n_circles > FrontWalls::kCircles;
+    for (int k = 0; k < g.n_circles; ++k)
+      if (crosses_seam(geo->circles[k], geo->nx, geo->ny)) w.everywhere = 1;
     w.n_circles = w.everywhere ? 0 : g.n_circles;
     for (int k = 0; k < w.n_circles; ++k) {
       w.cx[k] = (float)g.c[k].cx;

@@ -109,6 +109,19 @@ def test_walls_in_front_of_the_tiles_give_the_bits_of_the_wall_kernel(gpu_lib, p
             assert _same(_run([2, 1, 2], *args, 0, kind, circles, walls), apart), (scheme, walls)
 
 
+@pytest.mark.parametrize("precision,nx,ny,kind", [
+    (lbm.FP16_DEV, 1160, 1080, "cs"), (lbm.FP32_DEV, 700, 610, "none"), (lbm.FP64, 100, 90, "cs"),
+])
+def test_a_circle_round_the_fluid_may_cross_the_seam(gpu_lib, precision, nx, ny, kind):
+    # the fluid inside a circle that leaves the lattice on the left, or at a corner: boundary nodes all
+    # along the seam, far from the circle
+    for circle in ((0.34 * nx, 0.5 * ny, 0.52 * nx, 1), (0.26 * nx, 0.28 * ny, 0.43 * nx, 1)):
+        for scheme in ("bouzidi_q", "mod_b"):
+            args = (nx, ny, precision, scheme)
+            assert _same(_run([5], *args, 0, kind, [circle], False),
+                         _run([5], *args, 4 if nx > 100 else 1, kind, [circle], False)), scheme
+
+
 @pytest.mark.parametrize("precision", [lbm.FP64, lbm.FP32_DEV, lbm.FP16_DEV])
 @pytest.mark.parametrize("nx,ny", [(120, 64), (121, 75), (800, 500)])
 def test_channel_ends_in_the_tiles_give_the_bits_of_their_kernel(gpu_lib, precision, nx, ny):

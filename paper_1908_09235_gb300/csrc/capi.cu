@@ -995,11 +995,12 @@ lbm_status lbm_load_state(lbm_ctx* c, const void* buf, int64_t bytes) {
     LBM_CUDA(c, cudaMemcpyAsync(c->carry, in + sizeof(h) + c->lattice_bytes, 8 * c->nb,
                                 cudaMemcpyHostToDevice, c->stream));
   LBM_CUDA(c, cudaStreamSynchronize(c->stream));
-  const bool open_changed = (h.open_x != 0) != c->open_x;
+  const bool ends_changed =
+      (h.open_x != 0) != c->open_x || (c->open_x && std::memcmp(&h.u_in, &c->u_in, sizeof(double)) != 0);
   c->p.rho_ref = h.rho_ref;
   finalize_consts(c->p);
-  // captured steps hold the kernel parameters by value and the channel pass or not
-  if (c->p.rho_ref != c->graph_rho_ref || open_changed)
+  // captured steps hold the kernel parameters, the inflow velocity among them, by value
+  if (c->p.rho_ref != c->graph_rho_ref || ends_changed)
     for (int k = 0; k < 2; ++k)
       if (c->graph[k]) {
         cudaGraphExecDestroy(c->graph[k]);

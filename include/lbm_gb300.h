@@ -134,8 +134,8 @@ typedef struct {
                         *    and ny >= 8 (FP16: 12) the vectorised kernel (population vectors   *
                         *    of 16 B; the two psi-ring rows of tiles away from the x seam staged *
                         *    by tensor copies (TMA), the rest of the halo by cp.async), otherwise *
-                        *    the scalar tiles; a copy wait that expires is reported as           *
-                        *    LBM_ETIMEOUT by lbm_mass;                                           *
+                        *    the scalar tiles; a bounded wait that expires is reported as        *
+                        *    LBM_ETIMEOUT by the blocking reads;                                 *
                         * 1: the scalar tile kernel (one node per thread and row);              *
                         * 2: FP32 deviations on lattices with nx % 16 == 0, nx, ny >= 64: a     *
                         *    persistent kernel that stages tiles by TMA; otherwise as 0;         *
@@ -193,14 +193,17 @@ lbm_status lbm_step_timed(lbm_ctx* ctx, int32_t n, double* ms_step_kernel, doubl
 
 /* Total mass sum over fluid nodes and directions of f (FP64, fixed summation order, so repeated
  * calls on the same state agree bit for bit).  Blocks.  Returns LBM_EUNSTABLE (sticky) when a
- * fluid density is not finite or not positive. */
+ * fluid density is not finite or not positive, and as lbm_fields, lbm_force and lbm_save_state do
+ * LBM_ETIMEOUT (sticky) when a bounded wait of a step since the last initialisation or restored
+ * state gave up: that step went on without its data, and what is read is not the run's state. */
 lbm_status lbm_mass(lbm_ctx* ctx, double* out);
 
 /* Density and velocity (Eq. 5, with the half-force term) of every node into caller-owned host
  * arrays of nx*ny doubles; solid nodes get NaN.  Blocks. */
 lbm_status lbm_fields(lbm_ctx* ctx, double* rho, double* ux, double* uy);
 
-/* The same into device arrays of nx*ny doubles, asynchronously on the context's stream. */
+/* The same into device arrays of nx*ny doubles, asynchronously on the context's stream (so without
+ * the check for waits that gave up, which comes with the next blocking read). */
 lbm_status lbm_fields_device(lbm_ctx* ctx, double* rho, double* ux, double* uy);
 
 /* Node flags into a caller-owned host array of nx*ny bytes: bit 0 solid, bit 1 boundary node
@@ -265,6 +268,16 @@ lbm_status lbm_load_state(lbm_ctx* ctx, const void* buf, int64_t bytes);
  * LBM_EINVAL for a limit out of range. */
 lbm_status lbm_selftest_bounded_wait(int64_t limit_ns, int32_t complete, void* stream,
                                      int32_t* completed);
+
+/* Self-test of the wait of large lattices' tiles for the wall pass in front of them (and of its
+ * report): one thread waits on the context's stream for at most limit_ns nanoseconds (1 .. 1e10).
+ * complete != 0: there is nothing to wait for; LBM_OK with *completed = 1.  complete = 0: a count that
+ * nothing raises; the wait gives up, LBM_ETIMEOUT with *completed = 0, and the context is left as
+ * a step whose wait gave up leaves it: its next blocking read fails with LBM_ETIMEOUT, unless its
+ * state is set anew first.  The device stays usable either way.  Blocks.  LBM_EINVAL for a limit out
+ * of range. */
+lbm_status lbm_selftest_front_wait(lbm_ctx* ctx, int64_t limit_ns, int32_t complete,
+                                   int32_t* completed);
 
 /* Throughput of the GPU's FP64 fused multiply-add pipe, measured (measurement support; the
  * paper has no counterpart: the FP64 step of the method is bound by this pipe on GB300, and its

@@ -641,6 +641,16 @@ void lbm_destroy(lbm_ctx* c) {
   delete c;
 }
 
+// Waits for the work queued so far.  A bounded wait of a step that gave up (since the state was last
+// set) makes what was read invalid.
+static lbm_status finish_read(lbm_ctx* c) {
+  int err = 0;
+  LBM_CUDA(c, cudaMemcpyAsync(&err, c->err_flag, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+  LBM_CUDA(c, cudaStreamSynchronize(c->stream));
+  if (err & kErrTimeout) return fail(c, LBM_ETIMEOUT, "a bounded wait of a step kernel expired");
+  return LBM_OK;
+}
+
 static lbm_status init_common(lbm_ctx* c) {
   // captured steps hold the kernel parameters by value: keep them while rho_ref is unchanged
   if (c->p.rho_ref != c->graph_rho_ref)
@@ -653,6 +663,7 @@ static lbm_status init_common(lbm_ctx* c) {
                              c->stream));
   LBM_CUDA(c, cudaMemsetAsync(c->f[1], 0, c->lattice_bytes, c->stream));
   if (c->nb > 0) LBM_CUDA(c, cudaMemsetAsync(c->carry, 0, c->nb * 8, c->stream));
+  LBM_CUDA(c, cudaMemsetAsync(c->err_flag, 0, sizeof(int), c->stream));  // a new state
   LBM_CUDA(c, cudaStreamSynchronize(c->stream));
   c->cur = 0;
   c->steps = 0;
@@ -777,7 +788,7 @@ lbm_status lbm_mass(lbm_ctx* c, double* out) {
   LBM_CUDA(c, cudaMemcpyAsync(&err, c->err_flag, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
   LBM_CUDA(c, cudaStreamSynchronize(c->stream));
   *out = m;
-  if (err & kErrTimeout) return fail(c, LBM_ETIMEOUT, "a bounded wait for a tile copy expired");
+  if (err & kErrTimeout) return fail(c, LBM_ETIMEOUT, "a bounded wait of a step kernel expired");
   if (err) return fail(c, LBM_EUNSTABLE, "non-positive or non-finite density in the fluid");
   return LBM_OK;
 }
@@ -800,8 +811,7 @@ lbm_status lbm_fields(lbm_ctx* c, double* rho, double* ux, double* uy) {
   LBM_CUDA(c, cudaMemcpyAsync(rho, c->rho_m, N * 8, cudaMemcpyDeviceToHost, c->stream));
   LBM_CUDA(c, cudaMemcpyAsync(ux, c->ux_m, N * 8, cudaMemcpyDeviceToHost, c->stream));
   LBM_CUDA(c, cudaMemcpyAsync(uy, c->uy_m, N * 8, cudaMemcpyDeviceToHost, c->stream));
-  LBM_CUDA(c, cudaStreamSynchronize(c->stream));
-  return LBM_OK;
+  return finish_read(c);
 }
 
 lbm_status lbm_flags(lbm_ctx* c, uint8_t* flags) {
@@ -885,7 +895,8 @@ lbm_status lbm_force(lbm_ctx* c, double* fx, double* fy) {
     std::vector<double> h(2 * c->nb);
     LBM_CUDA(c, cudaMemcpyAsync(h.data(), c->force, c->nb * 16, cudaMemcpyDeviceToHost,
                                 c->stream));
-    LBM_CUDA(c, cudaStreamSynchronize(c->stream));
+    const lbm_status st = finish_read(c);
+    if (st != LBM_OK) return st;
     for (long long b = 0; b < c->nb; ++b) {  // boundary nodes in ascending order
       sx += h[2 * b];
       sy += h[2 * b + 1];
@@ -916,6 +927,19 @@ lbm_status lbm_selftest_bounded_wait(int64_t limit_ns, int32_t complete, void* s
   }
   *completed = h;
   return h == 1 ? LBM_OK : LBM_ETIMEOUT;
+}
+
+lbm_status lbm_selftest_front_wait(lbm_ctx* c, int64_t limit_ns, int32_t complete,
+                                   int32_t* completed) {
+  if (!c || !completed || limit_ns <= 0 || limit_ns > 10000000000LL) return LBM_EINVAL;
+  if (c->status) return c->status;
+  LBM_CUDA(c, launch_front_wait_selftest(c->front_done, complete ? 0 : 1, c->err_flag,
+                                         (unsigned long long)limit_ns, c->stream));
+  int err = 0;
+  LBM_CUDA(c, cudaMemcpyAsync(&err, c->err_flag, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+  LBM_CUDA(c, cudaStreamSynchronize(c->stream));
+  *completed = err & kErrTimeout ? 0 : 1;
+  return *completed ? LBM_OK : LBM_ETIMEOUT;
 }
 
 namespace {
@@ -967,8 +991,7 @@ lbm_status lbm_save_state(lbm_ctx* c, void* buf, int64_t bytes) {
   if (c->nb > 0)
     LBM_CUDA(c, cudaMemcpyAsync(out + sizeof(h) + c->lattice_bytes, c->carry, 8 * c->nb,
                                 cudaMemcpyDeviceToHost, c->stream));
-  LBM_CUDA(c, cudaStreamSynchronize(c->stream));
-  return LBM_OK;
+  return finish_read(c);
 }
 
 lbm_status lbm_load_state(lbm_ctx* c, const void* buf, int64_t bytes) {
@@ -994,6 +1017,7 @@ lbm_status lbm_load_state(lbm_ctx* c, const void* buf, int64_t bytes) {
   if (c->nb > 0)
     LBM_CUDA(c, cudaMemcpyAsync(c->carry, in + sizeof(h) + c->lattice_bytes, 8 * c->nb,
                                 cudaMemcpyHostToDevice, c->stream));
+  LBM_CUDA(c, cudaMemsetAsync(c->err_flag, 0, sizeof(int), c->stream));  // a new state
   LBM_CUDA(c, cudaStreamSynchronize(c->stream));
   const bool ends_changed =
       (h.open_x != 0) != c->open_x || (c->open_x && std::memcmp(&h.u_in, &c->u_in, sizeof(double)) != 0);

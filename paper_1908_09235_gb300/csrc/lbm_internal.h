@@ -114,6 +114,9 @@ bool step_march_supported(int precision, int eos, int nx, int ny);
 cudaError_t launch_step_march(const DevParams& p, const void* fa, void* fb, const uint8_t* flags,
                               double* rho_m, double* ux_m, double* uy_m, int* err, cudaStream_t s,
                               const FrontWalls* front = nullptr);
+// one thread waits, as a tile of the front does, for target counts of *done
+cudaError_t launch_front_wait_selftest(int* done, int target, int* err, unsigned long long limit_ns,
+                                       cudaStream_t s);
 // The step with the front, by the marching kernel or (FP32 single phase) the vector kernel; front: its
 // rows and CTA counts are filled in here.
 bool step_front_supported(int precision, int eos, int nx, int ny);

@@ -296,6 +296,12 @@ __global__ void __launch_bounds__(32, kWarps)
   if (__any_sync(0xffffffffu, !ok) && lane == 0) atomicOr(err, kErrTimeout);
 }
 
+// Self-test of the front's wait: one thread waits for w.ctas counts of w.done.
+__global__ void front_wait_selftest_kernel(const __grid_constant__ FrontWalls w, int* err,
+                                           unsigned long long limit_ns) {
+  wall::front_wait(w, err, limit_ns);
+}
+
 template <int EOS>
 cudaError_t launch_march_t(const DevParams& p, const void* fa, void* fb, const uint8_t* flags,
                            double* rho_m, double* ux_m, double* uy_m, int* err, cudaStream_t s,
@@ -322,6 +328,15 @@ cudaError_t launch_march_t(const DevParams& p, const void* fa, void* fb, const u
 bool step_march_supported(int precision, int eos, int nx, int ny) {
   return precision == LBM_FP16_DEV && eos != LBM_EOS_NONE && nx % 8 == 0 &&
          (long long)nx * ny > 152LL * 8192;
+}
+
+cudaError_t launch_front_wait_selftest(int* done, int target, int* err, unsigned long long limit_ns,
+                                       cudaStream_t s) {
+  FrontWalls w{};
+  w.done = done;
+  w.ctas = target;
+  front_wait_selftest_kernel<<<1, 1, 0, s>>>(w, err, limit_ns);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_step_march(const DevParams& p, const void* fa, void* fb, const uint8_t* flags,

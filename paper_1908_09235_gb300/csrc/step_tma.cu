@@ -7,7 +7,7 @@
 // the current one is computed.  Tiles that touch the periodic seam (whose ring wraps) are staged
 // with plain loads instead.  Every mbarrier wait is bounded (about 2 s): on expiry the CTA
 // records an error (kErrTimeout in the context's error word, reported as LBM_ETIMEOUT by
-// lbm_mass), waits boundedly for its own copies in flight and returns.
+// the blocking reads), waits boundedly for its own copies in flight and returns.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 

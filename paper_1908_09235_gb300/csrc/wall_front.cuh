@@ -61,10 +61,13 @@ __device__ __forceinline__ bool front_touches(const FrontWalls& w, int x0, int y
   return hit;
 }
 
-// One thread waits until the front is done; the caller's barrier comes after.  At most about 0.2 s,
-// and not at all once a wait of any tile has given up: that sets kErrTimeout in *err.
-constexpr unsigned long long kFrontWaitNs = 200000000ull;
-__device__ __forceinline__ void front_wait(const FrontWalls& w, int* err) {
+// One thread waits until the front is done; the caller's barrier comes after.  At most about limit_ns
+// (that of every bounded wait: a front has microseconds of work, but another process's time slice may
+// come between), and not at all once a wait of any tile has given up: that sets kErrTimeout in *err,
+// which fails the lattice's next blocking read (lbm_mass, lbm_fields, lbm_force, lbm_save_state), since
+// the tile goes on without the walls.
+__device__ __forceinline__ void front_wait(const FrontWalls& w, int* err,
+                                           unsigned long long limit_ns = tma::kWaitNs) {
   const unsigned long long t0 = tma::global_ns();
   for (long long i = 0; i < (1LL << 32); ++i) {
     int v;
@@ -72,7 +75,7 @@ __device__ __forceinline__ void front_wait(const FrontWalls& w, int* err) {
     if (v >= w.ctas) break;
     if ((i & 63) == 63) {
       if (*reinterpret_cast<volatile int*>(err) & kErrTimeout) break;
-      if (tma::global_ns() - t0 > kFrontWaitNs) {
+      if (tma::global_ns() - t0 > limit_ns) {
         atomicOr(err, kErrTimeout);
         break;
       }

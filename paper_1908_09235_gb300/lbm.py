@@ -35,7 +35,7 @@ EXPORTS = ("lbm_create", "lbm_coexistence", "lbm_init_fields", "lbm_init_droplet
            "lbm_batch_last_error", "lbm_batch_destroy", "lbm_batch_poll", "lbm_set_inflow",
            "lbm_force", "lbm_batch_tune_trials", "lbm_batch_set_schedule", "lbm_state_bytes",
            "lbm_save_state", "lbm_load_state", "lbm_selftest_bounded_wait",
-           "lbm_probe_fp64_fma")
+           "lbm_selftest_front_wait", "lbm_probe_fp64_fma")
 
 # lbm_schedule: how the CTAs of a batch's step kernel take tiles from its queue
 SCHED_STRIDED, SCHED_CLAIM, SCHED_CLAIM_LARGEST_FIRST = 0, 1, 2
@@ -168,6 +168,7 @@ def load_library(build_if_missing=True):
             "lbm_load_state": (C.c_int, [P, C.c_void_p, C.c_int64]),
             "lbm_selftest_bounded_wait": (C.c_int, [C.c_int64, C.c_int32, C.c_void_p,
                                                     C.POINTER(C.c_int32)]),
+            "lbm_selftest_front_wait": (C.c_int, [P, C.c_int64, C.c_int32, C.POINTER(C.c_int32)]),
             "lbm_probe_fp64_fma": (C.c_int, [C.c_int32, C.c_void_p, D, D]),
         }
         for name, (res, args) in sig.items():
@@ -291,6 +292,14 @@ def lbm_selftest_bounded_wait(limit_ns, complete, stream=None):
     done = C.c_int32(-1)
     st = load_library().lbm_selftest_bounded_wait(int(limit_ns), int(complete),
                                                   C.c_void_p(int(stream)), C.byref(done))
+    return st, done.value
+
+
+def lbm_selftest_front_wait(ctx, limit_ns, complete):
+    """(status, completed) of the front-wait self-test on a context (status 5, LBM_ETIMEOUT, when the
+    wait gave up); see include/lbm_gb300.h."""
+    done = C.c_int32(-1)
+    st = load_library().lbm_selftest_front_wait(ctx, int(limit_ns), int(complete), C.byref(done))
     return st, done.value
 
 

@@ -543,7 +543,9 @@ lbm_status lbm::create_context(const lbm_geometry* geo, const lbm_eos* eos, doub
   for (size_t k = 0; k < N; ++k) nf += (hf[k] & FLAG_SOLID) ? 0 : 1;
   c->n_fluid = nf;
 
-  // ---- third allocation: the wall pass within the step kernels ----
+  // ---- third allocation: the wall pass within the step kernels.  A lattice also runs without it, so
+  // where this memory is not to be had (the tables, and for FP64 24 bytes a node) its wall pass stays a
+  // launch of its own ----
   if (shape >= 0) {
     const TileTables tt((int)c->nb, h_bnode.data(), h_boff.data(), h_ldir.data(), geo->nx, geo->ny,
                         tw, th, eos->kind != LBM_EOS_NONE);
@@ -556,41 +558,38 @@ lbm_status lbm::create_context(const lbm_geometry* geo, const lbm_eos* eos, doub
                           align_up(nn * sizeof(TileNode)) + 2 * align_up(nn * 4);
     void* base3 = dev_alloc(c, tables + align_up(tt.links * tile_link_bytes(precision)) +
                                    align_up(c->nb * 8) + nm);
-    if (!base3) {
-      release_all(c);
-      delete c;
-      return LBM_ENOMEM;
+    if (base3) {
+      Carver c3{(char*)base3};
+      int4* heads = c3.take<int4>(tt.heads.size());
+      TileNode* nodes = c3.take<TileNode>(nn);
+      int32_t* first = c3.take<int32_t>(nn);
+      int32_t* local = c3.take<int32_t>(nn);
+      void* links = c3.take<char>(tt.links * tile_link_bytes(precision));
+      c->carry2 = c3.take<double>(c->nb);
+      // the deviation formats store FP32 moments: the second set fits behind the first
+      double* set0[3] = {c->rho_m, c->ux_m, c->uy_m};
+      for (int k = 0; k < 3; ++k)
+        c->macro2[k] = precision == LBM_FP64 ? c3.take<double>(N)
+                                             : reinterpret_cast<double*>((float*)set0[k] + N);
+      std::vector<char> up(tables);  // one upload
+      auto at = [&](const void* dev) { return up.data() + ((const char*)dev - (char*)base3); };
+      std::memcpy(at(heads), tt.heads.data(), tt.heads.size() * sizeof(int4));
+      std::memcpy(at(nodes), tt.nodes.data(), nn * sizeof(TileNode));
+      std::memcpy(at(first), tt.first.data(), nn * 4);
+      std::memcpy(at(local), tt.local.data(), nn * 4);
+      e = cudaMemcpyAsync(base3, up.data(), tables, cudaMemcpyHostToDevice, c->stream);
+      if (e == cudaSuccess)
+        e = launch_tile_links(precision, (int)nn, nodes, first, local, c->boff, c->ldir, c->recipe,
+                              links, c->stream);
+      if (e != cudaSuccess) return bail(e, "tile tables");
+      c->tiles.heads = heads;
+      c->tiles.nodes = nodes;
+      c->tiles.links = links;
+      c->tiles.max_links = tt.max_links;
+      c->tiles.max_nodes = tt.max_nodes;
+      c->tiles.cells = (tw + 2) * (th + 2);
+      c->tiles_shape = fits ? shape : -1;
     }
-    Carver c3{(char*)base3};
-    int4* heads = c3.take<int4>(tt.heads.size());
-    TileNode* nodes = c3.take<TileNode>(nn);
-    int32_t* first = c3.take<int32_t>(nn);
-    int32_t* local = c3.take<int32_t>(nn);
-    void* links = c3.take<char>(tt.links * tile_link_bytes(precision));
-    c->carry2 = c3.take<double>(c->nb);
-    // the deviation formats store FP32 moments: the second set fits behind the first
-    double* set0[3] = {c->rho_m, c->ux_m, c->uy_m};
-    for (int k = 0; k < 3; ++k)
-      c->macro2[k] = precision == LBM_FP64 ? c3.take<double>(N)
-                                           : reinterpret_cast<double*>((float*)set0[k] + N);
-    std::vector<char> up(tables);  // one upload
-    auto at = [&](const void* dev) { return up.data() + ((const char*)dev - (char*)base3); };
-    std::memcpy(at(heads), tt.heads.data(), tt.heads.size() * sizeof(int4));
-    std::memcpy(at(nodes), tt.nodes.data(), nn * sizeof(TileNode));
-    std::memcpy(at(first), tt.first.data(), nn * 4);
-    std::memcpy(at(local), tt.local.data(), nn * 4);
-    e = cudaMemcpyAsync(base3, up.data(), tables, cudaMemcpyHostToDevice, c->stream);
-    if (e == cudaSuccess)
-      e = launch_tile_links(precision, (int)nn, nodes, first, local, c->boff, c->ldir, c->recipe,
-                            links, c->stream);
-    if (e != cudaSuccess) return bail(e, "tile tables");
-    c->tiles.heads = heads;
-    c->tiles.nodes = nodes;
-    c->tiles.links = links;
-    c->tiles.max_links = tt.max_links;
-    c->tiles.max_nodes = tt.max_nodes;
-    c->tiles.cells = (tw + 2) * (th + 2);
-    c->tiles_shape = fits ? shape : -1;
   }
   // ---- large lattices: the wall pass in front of the step kernel's tiles ----
   if (!in_batch && shape < 0 && c->nb > 0 && !(opt && opt->kernel_path != 0) &&

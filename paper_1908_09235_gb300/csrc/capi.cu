@@ -518,9 +518,10 @@ lbm_status lbm::create_context(const lbm_geometry* geo, const lbm_eos* eos, doub
   // fluid node count (host, once), and the boundary list for the tables of the step kernels that do
   // the wall pass themselves
   int tw = 0, th = 0;
-  const int shape = in_batch || c->nb == 0 || (opt && opt->kernel_path != 0)
-                        ? -1
-                        : pick_step_tiles(precision, eos->kind, geo->nx, geo->ny, &tw, &th);
+  const bool walls_with_step =  // (see walls_in_steps)
+      !in_batch && c->nb > 0 && !(opt && opt->kernel_path != 0) && scheme != LBM_ZHAO_YONG;
+  const int shape =
+      walls_with_step ? pick_step_tiles(precision, eos->kind, geo->nx, geo->ny, &tw, &th) : -1;
   std::vector<uint8_t> hf(N), h_ldir;
   std::vector<int32_t> h_bnode, h_boff;
   if ((e = cudaMemcpyAsync(hf.data(), c->flags, N, cudaMemcpyDeviceToHost, c->stream)) !=
@@ -550,14 +551,16 @@ lbm_status lbm::create_context(const lbm_geometry* geo, const lbm_eos* eos, doub
     const TileTables tt((int)c->nb, h_bnode.data(), h_boff.data(), h_ldir.data(), geo->nx, geo->ny,
                         tw, th, eos->kind != LBM_EOS_NONE);
     // the tile's tables in shared memory (beside psi, within the 48 KB of a plain launch); a geometry
-    // with more walls in a tile than that keeps the wall pass apart
+    // with more walls in a tile than that keeps the wall pass apart (16 bodies in a 32 x 32 tile can
+    // take 57 KB)
     const size_t smem = 16u * tt.max_links + 10 * 8 * (size_t)tt.max_nodes + 4 * (tw + 2) * (th + 2);
     const bool fits = smem + 64 <= 40 * 1024;
     const size_t nn = tt.nodes.size(), nm = precision == LBM_FP64 ? 3 * align_up(N * 8) : 0;
     const size_t tables = align_up(tt.heads.size() * sizeof(int4)) +
                           align_up(nn * sizeof(TileNode)) + 2 * align_up(nn * 4);
-    void* base3 = dev_alloc(c, tables + align_up(tt.links * tile_link_bytes(precision)) +
-                                   align_up(c->nb * 8) + nm);
+    void* base3 = fits ? dev_alloc(c, tables + align_up(tt.links * tile_link_bytes(precision)) +
+                                          align_up(c->nb * 8) + nm)
+                       : nullptr;
     if (base3) {
       Carver c3{(char*)base3};
       int4* heads = c3.take<int4>(tt.heads.size());
@@ -588,11 +591,11 @@ lbm_status lbm::create_context(const lbm_geometry* geo, const lbm_eos* eos, doub
       c->tiles.max_links = tt.max_links;
       c->tiles.max_nodes = tt.max_nodes;
       c->tiles.cells = (tw + 2) * (th + 2);
-      c->tiles_shape = fits ? shape : -1;
+      c->tiles_shape = shape;
     }
   }
   // ---- large lattices: the wall pass in front of the step kernel's tiles ----
-  if (!in_batch && shape < 0 && c->nb > 0 && !(opt && opt->kernel_path != 0) &&
+  if (walls_with_step && shape < 0 &&
       step_front_supported(precision, eos->kind, geo->nx, geo->ny)) {
     c->front = true;
     for (int k = 0; k < 3; ++k) {

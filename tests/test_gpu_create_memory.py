@@ -42,3 +42,17 @@ def test_a_lattice_without_memory_for_the_tables_runs_with_the_wall_pass_apart(g
     mem = FailingMemory(3)
     assert _same(_run(_lattice(96, 64, precision, memory=mem)), want)
     assert mem.calls == 3 and not mem.live
+
+
+@pytest.mark.parametrize("nx,ny,scheme,circles", [
+    (96, 64, "zhao_yong", None),  # its wall pass reads the lattice that the next step overwrites
+    # 16 bodies in one 32 x 32 tile: its tables would take 57 KB of shared memory
+    (1301, 1000, "mod_a", [(66.3 + 8.5 * i, 66.1 + 8.5 * j, 3.25) for i in range(4) for j in range(4)]),
+])
+def test_tables_that_no_step_uses_take_no_memory(gpu_lib, nx, ny, scheme, circles):
+    def make(path):
+        return _lattice(nx, ny, lbm.FP32_DEV, scheme, circles, path=path)
+
+    here, apart = make(0), make(1)
+    assert here.info()["device_bytes"] == apart.info()["device_bytes"]
+    assert _same(_run(here, 5), _run(apart, 5))

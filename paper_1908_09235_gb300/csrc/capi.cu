@@ -481,6 +481,7 @@ lbm_status lbm::create_context(const lbm_geometry* geo, const lbm_eos* eos, doub
   c->nb = tot[0];
   c->nl = tot[1];
 
+  const int32_t last = (int32_t)c->nl;  // copied below; alive until the next synchronisation
   // ---- second allocation: boundary-link CSR and the FP64 rounding carry ----
   if (c->nb > 0) {
     size_t b2 = align_up(c->nb * 4) + align_up((c->nb + 1) * 4) + align_up(c->nl) +
@@ -503,7 +504,6 @@ lbm_status lbm::create_context(const lbm_geometry* geo, const lbm_eos* eos, doub
     if ((e = launch_geom_emit(g, c->flags, c->geom_tmp, c->bnode, c->boff, c->ldir, c->lq,
                               c->stream)) != cudaSuccess)
       return bail(e, "geom emit");
-    int32_t last = (int32_t)c->nl;
     if ((e = cudaMemcpyAsync(c->boff + c->nb, &last, 4, cudaMemcpyHostToDevice, c->stream)) !=
         cudaSuccess)
       return bail(e, "copy boff");
@@ -543,6 +543,11 @@ lbm_status lbm::create_context(const lbm_geometry* geo, const lbm_eos* eos, doub
   long long nf = 0;
   for (size_t k = 0; k < N; ++k) nf += (hf[k] & FLAG_SOLID) ? 0 : 1;
   c->n_fluid = nf;
+
+  if ((e = cudaMemsetAsync(c->f[0], 0, c->lattice_bytes, c->stream)) != cudaSuccess)
+    return bail(e, "memset f0");
+  if ((e = cudaMemsetAsync(c->f[1], 0, c->lattice_bytes, c->stream)) != cudaSuccess)
+    return bail(e, "memset f1");
 
   // ---- third allocation: the wall pass within the step kernels.  A lattice also runs without it, so
   // where this memory is not to be had (the tables, and for FP64 24 bytes a node) its wall pass stays a
@@ -584,6 +589,8 @@ lbm_status lbm::create_context(const lbm_geometry* geo, const lbm_eos* eos, doub
       if (e == cudaSuccess)
         e = launch_tile_links(precision, (int)nn, nodes, first, local, c->boff, c->ldir, c->recipe,
                               links, c->stream);
+      // the copy may read `up` until it is done
+      if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
       if (e != cudaSuccess) return bail(e, "tile tables");
       c->tiles.heads = heads;
       c->tiles.nodes = nodes;
@@ -621,10 +628,6 @@ lbm_status lbm::create_context(const lbm_geometry* geo, const lbm_eos* eos, doub
       w.r[k] = (float)g.c[k].r;
     }
   }
-  if ((e = cudaMemsetAsync(c->f[0], 0, c->lattice_bytes, c->stream)) != cudaSuccess)
-    return bail(e, "memset f0");
-  if ((e = cudaMemsetAsync(c->f[1], 0, c->lattice_bytes, c->stream)) != cudaSuccess)
-    return bail(e, "memset f1");
   c->kernel_path = opt ? opt->kernel_path : 0;
   c->track_force = opt && opt->track_force != 0;
   if (opt && opt->kernel_path == 2 && tma_step_supported(precision, geo->nx, geo->ny))

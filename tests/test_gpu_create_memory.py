@@ -56,3 +56,14 @@ def test_tables_that_no_step_uses_take_no_memory(gpu_lib, nx, ny, scheme, circle
     here, apart = make(0), make(1)
     assert here.info()["device_bytes"] == apart.info()["device_bytes"]
     assert _same(_run(here, 5), _run(apart, 5))
+
+
+def test_nothing_is_under_way_when_creation_with_tables_returns(gpu_lib):
+    # the tables are uploaded from host memory that is given back before lbm_create returns
+    import torch
+    s = torch.cuda.Stream()
+    lat = lbm.Lattice(1500, 1600, 1.0, "mod_a", circles=[(750.0, 560.0, 225.0)],
+                      eos=lbm.make_eos(lbm.EOS_NONE), precision=lbm.FP64, stream=s.cuda_stream)
+    idle = s.query()
+    lat.close()
+    assert idle

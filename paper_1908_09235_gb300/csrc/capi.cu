@@ -603,7 +603,7 @@ lbm_status lbm::create_context(const lbm_geometry* geo, const lbm_eos* eos, doub
   }
   // ---- large lattices: the wall pass in front of the step kernel's tiles ----
   if (walls_with_step && shape < 0 &&
-      step_front_supported(precision, eos->kind, geo->nx, geo->ny)) {
+      step_front_supported(precision, eos->kind, geo->nx, geo->ny, c->f[0], c->f[1])) {
     c->front = true;
     for (int k = 0; k < 3; ++k) {
       double* set0[3] = {c->rho_m, c->ux_m, c->uy_m};

@@ -109,17 +109,22 @@ cudaError_t launch_step(int precision, const DevParams& p, const void* fa, void*
                         bool fields_only, cudaStream_t s, int path = 0, int* err = nullptr);
 
 // The marching kernel of large two-phase FP16 lattices (csrc/step_march.cu); an expired wait sets
-// kErrTimeout in *err.
+// kErrTimeout in *err.  It needs tensor maps of its source lattice (a CUtensorMap each); where they
+// cannot be made (false) the vectorised kernel runs instead, in its form without tensor copies.
+struct alignas(64) MarchMaps {
+  unsigned char rest[128], moving[128];
+};
 bool step_march_supported(int precision, int eos, int nx, int ny);
-cudaError_t launch_step_march(const DevParams& p, const void* fa, void* fb, const uint8_t* flags,
+bool make_march_maps(MarchMaps* maps, const void* fa, int nx, int ny);
+cudaError_t launch_step_march(const MarchMaps& maps, const DevParams& p, const void* fa, void* fb, const uint8_t* flags,
                               double* rho_m, double* ux_m, double* uy_m, int* err, cudaStream_t s,
                               const FrontWalls* front = nullptr);
 // one thread waits, as a tile of the front does, for target counts of *done
 cudaError_t launch_front_wait_selftest(int* done, int target, int* err, unsigned long long limit_ns,
                                        cudaStream_t s);
 // The step with the front, by the marching kernel or (FP32 single phase) the vector kernel; front: its
-// rows and CTA counts are filled in here.
-bool step_front_supported(int precision, int eos, int nx, int ny);
+// rows and CTA counts are filled in here.  f0, f1: the two lattices, each the source in its turn.
+bool step_front_supported(int precision, int eos, int nx, int ny, const void* f0, const void* f1);
 cudaError_t launch_step_front(int precision, const DevParams& p, const void* fa, void* fb,
                               const uint8_t* flags, double* rho_m, double* ux_m, double* uy_m,
                               FrontWalls front, int* err, cudaStream_t s);

@@ -301,17 +301,21 @@ cudaError_t launch_step_tiles(int shape, int precision, const DevParams& p, cons
   return launch_tiles_s<double>(shape, p, fa, fb, flags, rho_m, ux_m, uy_m, wi, s);
 }
 
-bool step_front_supported(int precision, int eos, int nx, int ny) {
-  return step_march_supported(precision, eos, nx, ny) ||
-         (precision == LBM_FP32_DEV && eos == LBM_EOS_NONE &&
-          step_vec_supported(precision, nx, ny));
+bool step_front_supported(int precision, int eos, int nx, int ny, const void* f0, const void* f1) {
+  MarchMaps maps;
+  if (step_march_supported(precision, eos, nx, ny))
+    return make_march_maps(&maps, f0, nx, ny) && make_march_maps(&maps, f1, nx, ny);
+  return precision == LBM_FP32_DEV && eos == LBM_EOS_NONE && step_vec_supported(precision, nx, ny);
 }
 
 cudaError_t launch_step_front(int precision, const DevParams& p, const void* fa, void* fb,
                               const uint8_t* flags, double* rho_m, double* ux_m, double* uy_m,
                               FrontWalls front, int* err, cudaStream_t s) {
-  if (step_march_supported(precision, p.eos, p.nx, p.ny))
-    return launch_step_march(p, fa, fb, flags, rho_m, ux_m, uy_m, err, s, &front);
+  if (step_march_supported(precision, p.eos, p.nx, p.ny)) {
+    MarchMaps maps;
+    if (!make_march_maps(&maps, fa, p.nx, p.ny)) return cudaErrorNotSupported;
+    return launch_step_march(maps, p, fa, fb, flags, rho_m, ux_m, uy_m, err, s, &front);
+  }
   return launch_step_vec(precision, p, fa, fb, flags, rho_m, ux_m, uy_m, false, s, true, err,
                          &front);
 }
@@ -319,9 +323,11 @@ cudaError_t launch_step_front(int precision, const DevParams& p, const void* fa,
 cudaError_t launch_step(int precision, const DevParams& p, const void* fa, void* fb,
                         const uint8_t* flags, double* rho_m, double* ux_m, double* uy_m,
                         bool fields_only, cudaStream_t s, int path, int* err) {
+  MarchMaps maps;
   if ((path == 0 || path == 4) && !fields_only && err &&
-      step_march_supported(precision, p.eos, p.nx, p.ny))
-    return launch_step_march(p, fa, fb, flags, rho_m, ux_m, uy_m, err, s);
+      step_march_supported(precision, p.eos, p.nx, p.ny) &&
+      make_march_maps(&maps, fa, p.nx, p.ny))
+    return launch_step_march(maps, p, fa, fb, flags, rho_m, ux_m, uy_m, err, s);
   // FP64 is bound by the FP64 pipe, where the scalar tiling (fewer ring psi per node) is faster
   const bool vec = path == 3 || ((path == 0 || path == 4) && precision != LBM_FP64);
   if (vec && step_vec_supported(precision, p.nx, p.ny))

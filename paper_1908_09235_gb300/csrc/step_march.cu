@@ -303,12 +303,11 @@ __global__ void front_wait_selftest_kernel(const __grid_constant__ FrontWalls w,
 }
 
 template <int EOS>
-cudaError_t launch_march_t(const DevParams& p, const void* fa, void* fb, const uint8_t* flags,
+cudaError_t launch_march_t(const MarchMaps& maps, const DevParams& p, const void* fa, void* fb, const uint8_t* flags,
                            double* rho_m, double* ux_m, double* uy_m, int* err, cudaStream_t s,
                            const FrontWalls* front) {
-  CUtensorMap map{}, map2{};
-  if (!make_ring_tensor_maps_fp16(&map, &map2, fa, p.nx, p.ny, SWD, SWD))
-    return cudaErrorNotSupported;
+  const CUtensorMap& map = *reinterpret_cast<const CUtensorMap*>(maps.rest);
+  const CUtensorMap& map2 = *reinterpret_cast<const CUtensorMap*>(maps.moving);
   dim3 grid((p.nx + SWD - 1) / SWD, (p.ny + kRows - 1) / kRows);
   if (!front)
     return launch_pdl(step_march_kernel<EOS, false>, grid, dim3(32), s, p, fa, fb, flags,
@@ -339,12 +338,17 @@ cudaError_t launch_front_wait_selftest(int* done, int target, int* err, unsigned
   return cudaGetLastError();
 }
 
-cudaError_t launch_step_march(const DevParams& p, const void* fa, void* fb, const uint8_t* flags,
+bool make_march_maps(MarchMaps* maps, const void* fa, int nx, int ny) {
+  static_assert(sizeof(MarchMaps) == 2 * sizeof(CUtensorMap), "a tensor map each");
+  return make_ring_tensor_maps_fp16(maps->rest, maps->moving, fa, nx, ny, SWD, SWD);
+}
+
+cudaError_t launch_step_march(const MarchMaps& maps, const DevParams& p, const void* fa, void* fb, const uint8_t* flags,
                               double* rho_m, double* ux_m, double* uy_m, int* err, cudaStream_t s,
                               const FrontWalls* front) {
   if (p.eos == LBM_EOS_EXP)
-    return launch_march_t<LBM_EOS_EXP>(p, fa, fb, flags, rho_m, ux_m, uy_m, err, s, front);
-  return launch_march_t<LBM_EOS_CS>(p, fa, fb, flags, rho_m, ux_m, uy_m, err, s, front);
+    return launch_march_t<LBM_EOS_EXP>(maps, p, fa, fb, flags, rho_m, ux_m, uy_m, err, s, front);
+  return launch_march_t<LBM_EOS_CS>(maps, p, fa, fb, flags, rho_m, ux_m, uy_m, err, s, front);
 }
 
 }  // namespace lbm

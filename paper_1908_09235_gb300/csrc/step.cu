@@ -151,21 +151,30 @@ struct TileShape {
 };
 constexpr TileShape kShapes[] = {{16, 4, 1, 1}, {16, 8, 1, 1}, {32, 8, 1, 1},
                                  {32, 8, 1, 2}, {32, 8, 2, 2}, {32, 8, 4, 2}};
+// Whether pick_step_tiles gives shape k to lattices of a format with or without psi; the others are not
+// compiled.
+template <typename S, int EOS>
+constexpr bool shape_taken(int k) {
+  constexpr bool psi = EOS != LBM_EOS_NONE;
+  if (sizeof(S) == 8) return k == 0 || k == 1 || (psi && k == 4);
+  return k == 2 || (psi && k == 3) || k == 4 || (sizeof(S) == 4 && k == 5);
+}
 
 template <typename S, int EOS>
 cudaError_t launch_tiles_t(int shape, const DevParams& p, const void* fa, void* fb,
                            const uint8_t* flags, double* rho_m, double* ux_m, double* uy_m,
                            const WallIn* wi, cudaStream_t s) {
-#define LBM_SHAPE(k)                                                                         \
-  if (shape == k)                                                                            \
-  return launch_wall_shape<S, EOS, kShapes[k].w, kShapes[k].ty, kShapes[k].ry, kShapes[k].mode>( \
-      p, fa, fb, flags, rho_m, ux_m, uy_m, wi, s)
+#define LBM_SHAPE(k)                                                                           \
+  if constexpr (shape_taken<S, EOS>(k))                                                        \
+    if (shape == k)                                                                            \
+      return launch_wall_shape<S, EOS, kShapes[k].w, kShapes[k].ty, kShapes[k].ry, kShapes[k].mode>( \
+          p, fa, fb, flags, rho_m, ux_m, uy_m, wi, s)
   LBM_SHAPE(0);
   LBM_SHAPE(1);
   LBM_SHAPE(2);
   LBM_SHAPE(3);
   LBM_SHAPE(4);
-  if constexpr (sizeof(typename Pop<S>::C) == 4) LBM_SHAPE(5);
+  LBM_SHAPE(5);
 #undef LBM_SHAPE
   return cudaErrorInvalidValue;
 }

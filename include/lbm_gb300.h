@@ -125,20 +125,22 @@ typedef struct {
                         * initial fluid density, set by lbm_init_fields / lbm_init_droplet.     *
                         * Used rounded to the nearest FP32 value                                */
   int32_t kernel_path; /* step kernel, all with the same results bit for bit:                  *
-                        * 0: the fastest measured.  Small and mid-size lattices: scalar tiles   *
-                        *    sized to the lattice that also do the wall pass of the step before  *
-                        *    (the last step's stays a launch of its own; not for Zhao-Yong links *
-                        *    and some open channels).  Large two-phase FP16 lattices with        *
-                        *    nx % 8 == 0: a kernel whose warps march up strips of rows brought  *
-                        *    by tensor copies.  Others, with FP32/FP16 deviations, nx % 4 == 0 *
-                        *    and ny >= 8 (FP16: 12) the vectorised kernel (population vectors   *
-                        *    of 16 B; the two psi-ring rows of tiles away from the x seam staged *
-                        *    by tensor copies (TMA), the rest of the halo by cp.async), otherwise *
-                        *    the scalar tiles; a bounded wait that expires is reported as        *
-                        *    LBM_ETIMEOUT by the blocking reads;                                 *
+                        * 0: by size, format and model as measured.  Small and mid-size         *
+                        *    lattices: scalar tiles sized to the lattice that also do the wall  *
+                        *    pass of the step before (the last step's stays a launch of its     *
+                        *    own; not for Zhao-Yong links and some open channels, nor where the *
+                        *    device memory for its tables is not to be had).  Large two-phase   *
+                        *    FP16 lattices with nx % 8 == 0: a kernel whose warps march up      *
+                        *    strips of rows brought by tensor copies.  Others, with FP32/FP16   *
+                        *    deviations, nx % 4 == 0 and ny >= 8 (FP16: 12): the vectorised     *
+                        *    kernel (population vectors of 16 B; the two psi-ring rows of tiles *
+                        *    away from the x seam staged by tensor copies (TMA), the rest of    *
+                        *    the halo by cp.async).  Otherwise the scalar tiles.  A bounded     *
+                        *    wait that expires is reported as LBM_ETIMEOUT by the blocking      *
+                        *    reads;                                                             *
                         * 1: the scalar tile kernel (one node per thread and row);              *
                         * 2: FP32 deviations on lattices with nx % 16 == 0, nx, ny >= 64: a     *
-                        *    persistent kernel that stages tiles by TMA; otherwise as 0;         *
+                        *    persistent kernel that stages tiles by TMA; otherwise as 1;         *
                         * 3: the vectorised kernel wherever nx % 4 == 0 (FP64: nx % 2 == 0) and *
                         *    ny >= 8 (FP16: 12), FP64 included, its halo staged by cp.async     *
                         *    only; otherwise the scalar tiles;                                   *
@@ -187,7 +189,10 @@ lbm_status lbm_step(lbm_ctx* ctx, int32_t n);
 
 /* Advance n >= 1 steps without graphs, recording CUDA events around every kernel on the
  * context's stream; blocks until done and returns the summed milliseconds of the fused step
- * kernel, of the boundary kernel, and from the first event to the last.  Any pointer may be NULL. */
+ * kernel, of the boundary kernel, and from the first event to the last.  Any pointer may be NULL.
+ * The wall pass is a launch of its own here: where lbm_step has it inside the next step's kernel
+ * (lbm_options.kernel_path 0), other kernels are timed than lbm_step runs, those of kernel_path 4, with
+ * the same results. */
 lbm_status lbm_step_timed(lbm_ctx* ctx, int32_t n, double* ms_step_kernel, double* ms_boundary,
                           double* ms_total);
 

@@ -5,8 +5,8 @@
 // and goes through its rows one by one: psi of row y + 1 from the row just arrived, collision of row
 // y with psi of rows y - 1, y, y + 1 in registers, streaming of row y.  No CTA barrier stands between
 // loads and arithmetic, neighbours in x come by two shuffles per row, and there is no psi ring to
-// stage and index: 212 instructions per node against the vector kernel's 273, whose issue bounded the
-// FP16 step (40 B per node, 0.5 of HBM).  Rows arrive in kSlots shared-memory slots by tensor copies
+// stage and index: 222 thread instructions per fluid node (2048^2) against the vector kernel's 273, whose
+// issue bounded the FP16 step (40 B per node, 0.5 of HBM).  Rows arrive in kSlots shared-memory slots by tensor copies
 // (two per row, issued by one lane; every wait is bounded), so the loads in flight cost no registers.  psi of the columns
 // beside the strip is computed at the start, one (row, side) per lane.
 //

@@ -41,7 +41,8 @@ using namespace step_core;
 
 constexpr int VW = 32;  // lanes
 
-// async global -> shared copy of 8 or 16 bytes (both addresses aligned to the size), L2 only
+// async global -> shared copy of 8 or 16 bytes (both addresses aligned to the size): 16 bytes through L2
+// only; 8, and the 4 of the flags, also through L1 (why no old line is found there: d2q9.cuh, pdl_wait)
 __device__ __forceinline__ void cp_async(void* smem, const void* gmem, int bytes) {
   const uint32_t s = static_cast<uint32_t>(__cvta_generic_to_shared(smem));
   if (bytes == 16)

@@ -485,7 +485,7 @@ lbm_status lbm::create_context(const lbm_geometry* geo, const lbm_eos* eos, doub
   // ---- second allocation: boundary-link CSR and the FP64 rounding carry ----
   if (c->nb > 0) {
     size_t b2 = align_up(c->nb * 4) + align_up((c->nb + 1) * 4) + align_up(c->nl) +
-                align_up(c->nl * 8) + align_up(c->nb * 8) + align_up(c->nb * 16) +
+                align_up(c->nl * 8) + align_up(c->nb * 8) + align_up(c->nb * 16 + 8) +
                 align_up(link_recipe_bytes(c->nl));
     void* base2 = dev_alloc(c, b2);
     if (!base2) {
@@ -499,7 +499,10 @@ lbm_status lbm::create_context(const lbm_geometry* geo, const lbm_eos* eos, doub
     c->ldir = c2.take<uint8_t>(c->nl);
     c->lq = c2.take<double>(c->nl);
     c->carry = c2.take<double>(c->nb);
-    c->force = c2.take<double>(2 * c->nb);
+    // the error word moves behind the force, so that lbm_force reads both in one copy (4.1 ms of 200
+    // channel steps and their drag took 10 us longer with two)
+    c->force = c2.take<double>(2 * c->nb + 1);
+    c->err_flag = reinterpret_cast<int*>(c->force + 2 * c->nb);
     link_recipe_carve(c2.take<char>(link_recipe_bytes(c->nl)), c->nl, &c->recipe);
     if ((e = launch_geom_emit(g, c->flags, c->geom_tmp, c->bnode, c->boff, c->ldir, c->lq,
                               c->stream)) != cudaSuccess)
@@ -509,7 +512,7 @@ lbm_status lbm::create_context(const lbm_geometry* geo, const lbm_eos* eos, doub
       return bail(e, "copy boff");
     if ((e = cudaMemsetAsync(c->carry, 0, c->nb * 8, c->stream)) != cudaSuccess)
       return bail(e, "memset carry");
-    if ((e = cudaMemsetAsync(c->force, 0, c->nb * 16, c->stream)) != cudaSuccess)
+    if ((e = cudaMemsetAsync(c->force, 0, c->nb * 16 + 8, c->stream)) != cudaSuccess)
       return bail(e, "memset force");
     if ((e = launch_link_setup(c->p, (int)c->nb, c->bnode, c->boff, c->ldir, c->lq, c->flags,
                                c->recipe, c->stream)) != cudaSuccess)
@@ -646,14 +649,17 @@ void lbm_destroy(lbm_ctx* c) {
   delete c;
 }
 
-// Waits for the work queued so far.  A bounded wait of a step that gave up (since the state was last
-// set) makes what was read invalid.
+// A bounded wait of a step that gave up (since the state was last set) makes what was read invalid.
+static lbm_status check_waits(lbm_ctx* c, int err) {
+  return err & kErrTimeout ? fail(c, LBM_ETIMEOUT, "a bounded wait of a step kernel expired") : LBM_OK;
+}
+
+// Waits for the work queued so far.
 static lbm_status finish_read(lbm_ctx* c) {
   int err = 0;
   LBM_CUDA(c, cudaMemcpyAsync(&err, c->err_flag, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
   LBM_CUDA(c, cudaStreamSynchronize(c->stream));
-  if (err & kErrTimeout) return fail(c, LBM_ETIMEOUT, "a bounded wait of a step kernel expired");
-  return LBM_OK;
+  return check_waits(c, err);
 }
 
 static lbm_status init_common(lbm_ctx* c) {
@@ -793,7 +799,7 @@ lbm_status lbm_mass(lbm_ctx* c, double* out) {
   LBM_CUDA(c, cudaMemcpyAsync(&err, c->err_flag, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
   LBM_CUDA(c, cudaStreamSynchronize(c->stream));
   *out = m;
-  if (err & kErrTimeout) return fail(c, LBM_ETIMEOUT, "a bounded wait of a step kernel expired");
+  if (check_waits(c, err) != LBM_OK) return LBM_ETIMEOUT;
   if (err) return fail(c, LBM_EUNSTABLE, "non-positive or non-finite density in the fluid");
   return LBM_OK;
 }
@@ -897,10 +903,13 @@ lbm_status lbm_force(lbm_ctx* c, double* fx, double* fy) {
     return fail(c, LBM_ESTATE, "the force is not recorded (lbm_options.track_force)");
   double sx = 0.0, sy = 0.0;
   if (c->nb > 0) {
-    std::vector<double> h(2 * c->nb);
-    LBM_CUDA(c, cudaMemcpyAsync(h.data(), c->force, c->nb * 16, cudaMemcpyDeviceToHost,
+    std::vector<double> h(2 * c->nb + 1);
+    LBM_CUDA(c, cudaMemcpyAsync(h.data(), c->force, c->nb * 16 + 8, cudaMemcpyDeviceToHost,
                                 c->stream));
-    const lbm_status st = finish_read(c);
+    LBM_CUDA(c, cudaStreamSynchronize(c->stream));
+    int err;
+    std::memcpy(&err, &h[2 * c->nb], sizeof(int));
+    const lbm_status st = check_waits(c, err);
     if (st != LBM_OK) return st;
     for (long long b = 0; b < c->nb; ++b) {  // boundary nodes in ascending order
       sx += h[2 * b];

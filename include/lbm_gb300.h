@@ -277,8 +277,8 @@ lbm_status lbm_selftest_bounded_wait(int64_t limit_ns, int32_t complete, void* s
 /* Self-test of the wait of large lattices' tiles for the wall pass in front of them (and of its
  * report): one thread waits on the context's stream for at most limit_ns nanoseconds (1 .. 1e10).
  * complete != 0: there is nothing to wait for; LBM_OK with *completed = 1.  complete = 0: a count that
- * nothing raises; the wait gives up, LBM_ETIMEOUT with *completed = 0, and the context is left as
- * a step whose wait gave up leaves it: its next blocking read fails with LBM_ETIMEOUT, unless its
+ * nothing raises; the wait gives up, LBM_ETIMEOUT with *completed = 0, and the error word is left as
+ * an expired wait leaves it: after the next step a blocking read fails with LBM_ETIMEOUT, unless the
  * state is set anew first.  The device stays usable either way.  Blocks.  LBM_EINVAL for a limit out
  * of range. */
 lbm_status lbm_selftest_front_wait(lbm_ctx* ctx, int64_t limit_ns, int32_t complete,

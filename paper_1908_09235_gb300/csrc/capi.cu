@@ -651,11 +651,17 @@ void lbm_destroy(lbm_ctx* c) {
 
 // A bounded wait of a step that gave up (since the state was last set) makes what was read invalid.
 static lbm_status check_waits(lbm_ctx* c, int err) {
-  return err & kErrTimeout ? fail(c, LBM_ETIMEOUT, "a bounded wait of a step kernel expired") : LBM_OK;
+  if (err & kErrTimeout) return fail(c, LBM_ETIMEOUT, "a bounded wait of a step kernel expired");
+  c->waits_unread = false;
+  return LBM_OK;
 }
 
 // Waits for the work queued so far.
 static lbm_status finish_read(lbm_ctx* c) {
+  if (!c->waits_unread) {
+    LBM_CUDA(c, cudaStreamSynchronize(c->stream));
+    return LBM_OK;
+  }
   int err = 0;
   LBM_CUDA(c, cudaMemcpyAsync(&err, c->err_flag, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
   LBM_CUDA(c, cudaStreamSynchronize(c->stream));
@@ -676,6 +682,7 @@ static lbm_status init_common(lbm_ctx* c) {
   if (c->nb > 0) LBM_CUDA(c, cudaMemsetAsync(c->carry, 0, c->nb * 8, c->stream));
   LBM_CUDA(c, cudaMemsetAsync(c->err_flag, 0, sizeof(int), c->stream));  // a new state
   LBM_CUDA(c, cudaStreamSynchronize(c->stream));
+  c->waits_unread = false;
   c->cur = 0;
   c->steps = 0;
   c->initialized = true;
@@ -728,6 +735,7 @@ lbm_status lbm_step(lbm_ctx* c, int32_t n) {
   if (c->status) return c->status;
   if (n < 0) return LBM_EINVAL;
   if (!c->initialized) return fail(c, LBM_ESTATE, "lbm_step before initialisation");
+  c->waits_unread = c->waits_unread || n > 0;
   while (n >= c->graph_steps) {
     if (!c->graph[c->cur]) {
       lbm_status st = build_graph(c, c->cur);
@@ -750,6 +758,7 @@ lbm_status lbm_step_timed(lbm_ctx* c, int32_t n, double* ms_step, double* ms_bnd
   if (c->status) return c->status;
   if (n < 1) return LBM_EINVAL;
   if (!c->initialized) return fail(c, LBM_ESTATE, "lbm_step_timed before initialisation");
+  c->waits_unread = true;
   std::vector<cudaEvent_t> ev(2 * (size_t)n + 1);
   for (auto& e : ev) LBM_CUDA(c, cudaEventCreate(&e));
   lbm_status st = LBM_OK;
@@ -1047,6 +1056,7 @@ lbm_status lbm_load_state(lbm_ctx* c, const void* buf, int64_t bytes) {
   c->open_x = h.open_x != 0;
   c->u_in = h.u_in;
   if (c->open_x) c->track_force = true;
+  c->waits_unread = false;
   c->cur = 0;
   c->steps = h.steps;
   c->initialized = true;

@@ -355,6 +355,7 @@ struct lbm_ctx {
   double* partials = nullptr;
   double* mass_out = nullptr;
   int* err_flag = nullptr;
+  bool waits_unread = false;  // steps were launched since err_flag was last read (or cleared)
   int2* geom_tmp = nullptr;
   long long* geom_totals = nullptr;
   int ledger_blocks = 0;

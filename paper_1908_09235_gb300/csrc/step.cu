@@ -313,13 +313,13 @@ cudaError_t launch_step_tiles(int shape, int precision, const DevParams& p, cons
 // Every lattice of the marching kernel, and the single-phase FP32 ones that the vector kernel takes, at
 // every size the tiles above leave.  Single phase, us a step in front / apart, one cylinder of r = nx/80
 // (r = 0.15 of the side):
-//              640^2                     1000 x 625    1024^2                    1600 x 1000   2048^2
-//   closed     7.1 / 6.9 (7.6 / 7.1)     8.3 / 8.7     9.7 / 11.1 (11.3 / 11.3)  17.1 / 18.7   46.2 / 49.2
-//   channel    12.7 / 8.7 (13.8 / 9.4)   12.9 / 10.8   16.2 / 13.3 (19.0 / 13.5) 20.2 / 21.5   49.8 / 51.9
-// So a closed lattice gains from about 0.6 M nodes on, and a channel only from about 1.4 M: its inlet is
-// FP64 work of ny rows, which the front's few 256-thread CTAs do on as few SMs (by itself it runs in
-// one-warp CTAs).  Below that the rule is not the fastest; all of these are faster than three launches
-// in plain stream order (channels 15.5, 17.2, 20.1, 29.6, 60.2).
+//             640^2                   1024^2                    1600 x 1000               2048^2
+//   closed    7.1 / 6.9 (7.6 / 7.1)   9.7 / 11.1 (11.3 / 11.3)  17.1 / 18.7 (17.7 / 19.0) 46.2 / 49.2 (47.1 / 50.4)
+//   channel   12.7 / 8.7 (13.8 / 9.4) 16.2 / 13.3 (19.0 / 13.5) 20.2 / 21.5 (21.9 / 21.6) 49.8 / 51.9 (50.8 / 55.0)
+// So a closed lattice gains from about 0.6 M nodes on (large cylinder: 1 M), and a channel only from about
+// 1.5 M (large cylinder: between 2 and 4 M): its inlet is FP64 work of ny rows, which the front's few
+// 256-thread CTAs do on as few SMs (by itself it runs in one-warp CTAs).  Below that the rule is not the fastest; all of these are faster than three launches
+// in plain stream order (channels 15.5, 20.1, 29.6, 60.2).
 bool step_front_supported(int precision, int eos, int nx, int ny, const void* f0, const void* f1) {
   MarchMaps maps;
   if (step_march_supported(precision, eos, nx, ny))
